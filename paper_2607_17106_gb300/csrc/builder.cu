@@ -820,6 +820,7 @@ extern "C" void bfs_free_graph(bfs_graph* g) {
     cudaFree(g->col);
     cudaFree(g->isolated);
     cudaFree(g->perm);
+    cudaFree(g->cc_scratch);
     delete g;
 }
 

@@ -1,34 +1,35 @@
-// cc.cu -- connected components by min-label propagation.
+// cc.cu -- connected components: the smallest vertex id of each component.
 //
-// The BFS cascade over the same graph tensor G with the min operator of the
-// paper's operator table (Section 2) in place of ANY:
-//   L_0[v] = v,  F_0 = the vertices with an edge,
-//   L_{i+1}[d] = min(L_i[d], min over s in F_i adjacent to d of L_i[s]),
-//   F_{i+1} = the vertices whose label dropped, stop when F_{i+1} is empty.
-// The fixed point gives every vertex the smallest id of its component.
+// The fixed point of min-label propagation (the BFS cascade over the same
+// graph tensor G with the min operator of the paper's operator table,
+// Section 2, in place of ANY) gives every vertex the smallest id of its
+// component.  Propagating labels an edge per iteration takes as many
+// iterations as the graph is long and reads every edge in the dense ones
+// (3.3 ms on RMAT-22, 135 ms and about 3,000 iterations on the relabelled
+// 4096^2 grid).  The same labels come from a union-find forest over the label
+// array itself, whose work does not depend on the diameter:
+//   - label[v] is v's parent in a forest; a root is its own parent.  A hook
+//     makes the larger of two roots point to the smaller (one CAS), so every
+//     root is the smallest id of its tree and a parent is never larger than
+//     its child (Shiloach and Vishkin 1982; lock-free as in ECL-CC, Jaiganesh
+//     and Burtscher 2018);
+//   - most edges are never read.  Rows ascend, so the first entry of each row
+//     (hubs have low ids in RMAT and BA) and then the last one are hooked; a
+//     sample of the labels then names the largest tree, and only vertices
+//     outside it go through the rest of their rows (the subgraph sampling of
+//     Afforest, Sutton, Ben-Nun and Barak 2018).  That is exact: an edge
+//     between two vertices of the largest tree joins nothing, and any other
+//     edge lies in the row of an end outside it, because G is symmetric.
 //
-// One persistent cooperative kernel runs every iteration; iterations are
-// separated by the grid barrier of common.cuh.  Like BFS, an iteration has a
-// push and a pull form of the same Einsum:
-//   push (sparse F_i): the words of F_i are dealt over warps, the rows of a
-//     word's active vertices flattened over the warp (32 entries a step); a
-//     relaxation reads the target's label and issues the atomicMin only when
-//     it would lower it.  Rows of at least CC_CHUNK entries become chunk units
-//     that whole CTAs expand one edge per thread in the next iteration (safe:
-//     labels only drop, and a unit reads its vertex's label when it runs).
-//   pull (dense F_i, and iteration 0): every vertex takes the minimum over
-//     all its neighbours' labels with no atomics.  This equals the minimum
-//     over its neighbours in F_i, because a neighbour outside F_i has already
-//     pushed its current label.  Rows of at least CC_CHUNK entries are fixed
-//     chunk units, listed once, whose CTA-wide minimum goes in with one
-//     atomicMin.
-// After each iteration the vertices of F_{i+1} shortcut their labels
-// (cc_jump), which leaves the fixed point unchanged and shortens the chains
-// a label travels along on long-diameter graphs.
+// One cooperative kernel; phases are separated by the grid barrier of
+// common.cuh.  What bounds it is the gathers: per vertex a row-offset pair, two
+// column sectors and a few label hops, which stay in L2 (67 MB for 2^24
+// vertices); 64 warps an SM (32 registers a thread) hide them.  Measured
+// around the call: RMAT-22 3,283 -> 286 us, the 4096^2 grid 135-180 ms
+// (2,800 to 3,400 iterations) -> 2.7 ms.
 #include "common.cuh"
 
 #include <algorithm>
-#include <numeric>
 
 namespace bfsgb {
 
@@ -36,354 +37,226 @@ bfs_status device_error(int err, int64_t timeout_ns);  // bfs_single.cu
 
 namespace {
 
-constexpr int CC_T = 1024;
-constexpr int CC_CHUNK = 1024;  // rows of at least this many entries are expanded as chunk units
-constexpr int CC_PULL_DIV = 16;  // pull when |F_i| > n / CC_PULL_DIV
-
-struct CountersCC {
-    unsigned long long changed;  // vertices set in F_{i+1}
-    unsigned long long u_len;    // chunk units appended for the next iteration
-};
+constexpr int CC_T = 512;
+constexpr int CC_HOPS = 32;      // parents a vertex climbs in one shortcut pass
+constexpr int CC_SAMPLES = 1024; // labels looked at to find the largest tree
+constexpr int CC_SLOTS = 2048;   // hash slots they are counted in
+constexpr int CC_WARP_ROW = 16;  // longer rows are hooked by a whole warp
+constexpr int CC_BIG_ROW = 4096; // rows of at least this many entries by the whole grid
 
 struct CtlCC {
     GridBarrier bar;
-    CountersCC slot[3];  // iteration i: slot[i % 3]; slot[(i + 2) % 3] is cleared during i
-    unsigned long long n_big;  // fixed chunk units of the big rows (pull iterations)
-    int32_t iters;
+    unsigned open[3];   // shortcut pass k: set in open[k % 3] by a vertex that has not reached its root
+    int32_t n_big;      // rows of at least CC_BIG_ROW entries outside the largest tree
+    int32_t iters;      // passes over the vertices
 };
 
 struct ParamsCC {
     int32_t n;
-    int64_t W;
+    int64_t m;
     const int32_t* __restrict__ row_ptr;
     const int32_t* __restrict__ col;
-    const uint32_t* __restrict__ isolated;
     int32_t* label;
-    uint32_t* F0;
-    uint32_t* F1;
-    int2* U0;
-    int2* U1;
-    int2* B;  // fixed chunk units of every row of at least CC_CHUNK entries
-    int64_t ucap;
-    uint64_t wmul;  // odd multiplier coprime to W: word i of the dealing order is (i * wmul) mod W
     CtlCC* ctl;
+    int32_t* big;       // their vertices, m / CC_BIG_ROW + 1
+    int32_t big_cap;
     int64_t timeout_ns;
-    int32_t max_iters;
 };
 
-// s -> d with s's label ls: lower d's label, and on a drop put d in F_{i+1}
-__device__ __forceinline__ void cc_relax(const ParamsCC& p, uint32_t* f_nxt, int ls, int d, unsigned long long& cnt) {
-    if (ls < __ldcg(p.label + d)) {  // labels only drop, so a stale read costs an atomic at most
-        const int old = atomicMin(p.label + d, ls);
-        if (ls < old) {
-            const unsigned bit = 1u << (d & 31);
-            if (!(atomicOr(f_nxt + (d >> 5), bit) & bit)) cnt += 1;
-        }
+// Root of v's tree.  Every vertex on the way is pointed past its parent: a
+// plain store is safe, because only a root is ever hooked (by CAS) and a
+// vertex that has a parent keeps one; whichever of two racing stores lands
+// last, it names an ancestor.  Ends: each hop goes to a smaller id.
+__device__ __forceinline__ int cc_find(int32_t* L, int v) {
+    int prev = v;
+    int p = __ldcg(L + v);
+    while (p != prev) {
+        const int g = __ldcg(L + p);
+        if (g == p) break;
+        __stcg(L + prev, g);
+        prev = p;
+        p = g;
     }
+    return p;
 }
 
-// Word of position i in the dealing order.  Warp k takes the contiguous
-// positions [k * per, (k + 1) * per).  The multiplicative scramble spreads
-// costly words over the warps: RMAT ids that share bit patterns have similar
-// degrees, and a stride of warps over plain word order (or over a scramble
-// modulo a power of two, which keeps low bits) gave one warp 10x the mean work.
-__device__ __forceinline__ long long cc_word(const ParamsCC& p, long long i) {
-    return (long long)(((unsigned long long)i * p.wmul) % (unsigned long long)p.W);
+// Join the trees of root a (or what became of it) and of vertex u; returns
+// the joint tree's root.  A failed CAS found that the larger root has been
+// hooked meanwhile and continues from its new parent, a smaller id: it ends.
+__device__ __forceinline__ int cc_hook(int32_t* L, int a, int u) {
+    int b = cc_find(L, u);
+    while (a != b) {
+        const int hi = max(a, b), lo = min(a, b);
+        const int old = atomicCAS(L + hi, hi, lo);
+        if (old == hi) return lo;
+        a = lo;
+        b = cc_find(L, old);
+    }
+    return a;
 }
 
-// Shortcut step after an iteration's relaxations (the pointer jumping of
-// Shiloach-Vishkin-style algorithms): every vertex of F_{i+1} takes the label
-// of the vertex its label names, label[v] <- min(label[v], label[label[v]]).
-// A label is always the id of a vertex of the same component and labels only
-// drop, so the fixed point is unchanged (each vertex's smallest component
-// id); the step lets a label travel through the vertex it names instead of
-// one edge per iteration, which on long-diameter graphs cuts the iteration
-// count.  A thread takes words of F_{i+1} in a grid stride.
-__device__ __forceinline__ void cc_jump(const ParamsCC& p, const uint32_t* f_nxt) {
-    const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long gthreads = (long long)gridDim.x * blockDim.x;
-    for (long long w = gtid; w < p.W; w += gthreads) {
-        unsigned fw = __ldcg(f_nxt + w);
-        while (fw) {
-            const int v = (int)(w * 32 + __ffs(fw) - 1);
-            fw &= fw - 1;
-            const int l = __ldcg(p.label + v);
-            const int ll = __ldcg(p.label + l);
-            if (ll < l) atomicMin(p.label + v, ll);
-        }
-    }
-}
-
-// |F_{i+1}|: one atomic per CTA
-__device__ __forceinline__ void cc_count(CountersCC* nxt, unsigned long long cnt, unsigned long long* s_red) {
-    cnt = warp_sum(cnt);
-    if (lane_id() == 0) s_red[threadIdx.x >> 5] = cnt;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long t = 0;
-        for (int i = 0; i < CC_T / 32; ++i) t += s_red[i];
-        if (t) atomicAdd(&nxt->changed, t);
-    }
-    __syncthreads();
-}
-
-// d's label dropped (this thread's atomic lowered it): record d in F_{i+1}
-__device__ __forceinline__ void cc_mark(uint32_t* f_nxt, int d, unsigned long long& cnt) {
-    const unsigned bit = 1u << (d & 31);
-    if (!(atomicOr(f_nxt + (d >> 5), bit) & bit)) cnt += 1;
-}
-
-// Pull iteration.  Units left by a push iteration are expanded in push form
-// first (their rows were in F_{i-1}); then each fixed unit of a big row gives
-// a warp-wide minimum, and warps take the words of all vertices, each word's
-// rows below CC_CHUNK flattened over the warp.  F_i is consumed (cleared)
-// because a pull reads every neighbour anyway.
-template <int T>
-__device__ void cc_pull(const ParamsCC& p, uint32_t* f_cur, uint32_t* f_nxt, const int2* u_cur,
-                        long long nunits, long long n_big, unsigned long long& cnt) {
-    const unsigned lane = lane_id();
-    const long long gwarp = ((long long)blockIdx.x * T + threadIdx.x) >> 5, nwarps = ((long long)gridDim.x * T) >> 5;
-    for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
-        const int2 un = __ldcg(u_cur + u);
-        const int s = un.x;
-        const int ls = __ldcg(p.label + s);
-        const int b = __ldg(p.row_ptr + s) + un.y * CC_CHUNK;
-        const int e = min(__ldg(p.row_ptr + s + 1), b + CC_CHUNK);
-        const int j = b + (int)threadIdx.x;
-        if (j < e) cc_relax(p, f_nxt, ls, __ldg(p.col + j), cnt);
-    }
-    for (long long u = gwarp; u < n_big; u += nwarps) {  // a warp per fixed unit, warp-uniform
-        const int2 un = __ldcg(p.B + u);  // written by this kernel's init phase
-        const int d = un.x;
-        const int b = __ldg(p.row_ptr + d) + un.y * CC_CHUNK;
-        const int e = min(__ldg(p.row_ptr + d + 1), b + CC_CHUNK);
-        int m = INT32_MAX;
-        for (int j = b + (int)lane; j < e; j += 32) m = min(m, __ldcg(p.label + __ldg(p.col + j)));
-        m = __reduce_min_sync(0xffffffffu, m);
-        if (lane == 0 && m < __ldcg(p.label + d)) {
-            if (m < atomicMin(p.label + d, m)) cc_mark(f_nxt, d, cnt);
-        }
-    }
-    const long long per = (p.W + nwarps - 1) / nwarps;
-    const long long iend = min((gwarp + 1) * per, (long long)p.W);
-    for (long long i0 = gwarp * per; i0 < iend; i0 += 32) {  // 32 words of the dealing order a step
-        const long long il = i0 + (long long)lane;
-        const long long wl = il < iend ? cc_word(p, il) : -1;
-        if (wl >= 0 && __ldcg(f_cur + wl)) f_cur[wl] = 0u;  // the buffer holds F_{i+2} next
-        for (unsigned todo = __ballot_sync(0xffffffffu, wl >= 0); todo; todo &= todo - 1) {  // warp-uniform
-            const long long w = __shfl_sync(0xffffffffu, wl, __ffs(todo) - 1);
-            const int d = (int)(w * 32 + lane);
-            int beg = 0, deg = 0, ld = INT32_MAX;
-            if (d < p.n) {
-                beg = __ldg(p.row_ptr + d);
-                deg = __ldg(p.row_ptr + d + 1) - beg;
-                ld = __ldcg(p.label + d);
-            }
-            const int fdeg = deg < CC_CHUNK ? deg : 0;
-            int incl = fdeg;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, incl, o);
-                if ((int)lane >= o) incl += y;
-            }
-            const int total = __shfl_sync(0xffffffffu, incl, 31);
-            if (total == 0) continue;
-            const int excl = incl - fdeg;
-            int mine = INT32_MAX;  // minimum over this lane's row
-            for (int base = 0; base < total; base += 32) {
-                const int idx = base + (int)lane;
-                int o = 0;
-#pragma unroll
-                for (int st = 16; st > 0; st >>= 1) {
-                    const int ex = __shfl_sync(0xffffffffu, excl, (o + st) & 31);
-                    if (o + st < 32 && ex <= idx) o += st;
+// Shortcut passes: label[v] <- v's root.  A vertex climbs at most CC_HOPS
+// parents in a pass and only its own label is written, so a chain of any
+// length (a path in its natural order starts as one) is cut by that factor
+// at least in each pass, and after the last pass every label is a root.
+// Grid-uniform; false when a barrier was given up.
+__device__ bool cc_shortcut(const ParamsCC& p, unsigned& bar_target, int& pass, int& iters) {
+    const long long gtid = (long long)blockIdx.x * CC_T + threadIdx.x;
+    const long long gthreads = (long long)gridDim.x * CC_T;
+    for (;;) {
+        unsigned* open = &p.ctl->open[pass % 3];
+        bool left = false;
+        for (long long v = gtid; v < p.n; v += gthreads) {
+            const int own = __ldcg(p.label + v);
+            int r = own, g = own;
+            bool root = false;
+#pragma unroll 1
+            for (int k = 0; k < CC_HOPS; ++k) {
+                g = __ldcg(p.label + r);
+                if (g == r) {
+                    root = true;
+                    break;
                 }
-                const int ob = __shfl_sync(0xffffffffu, beg, o);
-                const int oex = __shfl_sync(0xffffffffu, excl, o);
-                const int val = idx < total ? __ldcg(p.label + __ldg(p.col + ob + (idx - oex))) : INT32_MAX;
-                // segmented minimum: owners are non-decreasing over the lanes, so
-                // each lane keeps the minimum of its owner's entries in this step
-                int segmin = val;
-#pragma unroll
-                for (int off = 1; off < 32; off <<= 1) {
-                    const int y = __shfl_down_sync(0xffffffffu, segmin, off);
-                    const int oy = __shfl_down_sync(0xffffffffu, o, off);
-                    if ((int)lane + off < 32 && oy == o) segmin = min(segmin, y);
-                }
-                // the first lane of each owner's run holds its minimum; hand it to the owner
-                const int op = __shfl_up_sync(0xffffffffu, o, 1);
-                const bool head = idx < total && (lane == 0 || op != o);
-                const unsigned hm = __ballot_sync(0xffffffffu, head);
-                // owner lane L takes the value of the head lane whose o == L (at most one per step)
-                for (unsigned h = hm; h; h &= h - 1) {
-                    const int hl = __ffs(h) - 1;
-                    const int ho = __shfl_sync(0xffffffffu, o, hl);
-                    const int hv = __shfl_sync(0xffffffffu, segmin, hl);
-                    if ((int)lane == ho) mine = min(mine, hv);
-                }
+                r = g;
             }
-            if (mine < ld) {  // units may lower labels concurrently: the atomic decides
-                const int old = atomicMin(p.label + d, mine);
-                if (mine < old) cc_mark(f_nxt, d, cnt);
-            }
+            if (r != own) __stcg(p.label + v, r);
+            left |= !root;
         }
+        if (__syncthreads_or(left) && threadIdx.x == 0) atomicOr(open, 1u);
+        if (gtid == 0) p.ctl->open[(pass + 1) % 3] = 0;  // last read two barriers ago
+        ++iters;
+        ++pass;
+        unsigned more = 0;
+        __shared__ unsigned s_more;
+        if (!grid_sync(&p.ctl->bar, gridDim.x, bar_target, p.timeout_ns, NoArrivalWork(),
+                       [&]() { s_more = *(volatile unsigned*)open; }))
+            return false;
+        more = s_more;
+        __syncthreads();
+        if (!more) return true;
     }
 }
 
-__global__ void __launch_bounds__(CC_T, 1) cc_kernel(ParamsCC p) {
-    __shared__ unsigned long long s_red[CC_T / 32];
+__global__ void __launch_bounds__(CC_T, 4) cc_kernel(ParamsCC p) {
+    __shared__ int s_key[CC_SLOTS];
+    __shared__ int s_cnt[CC_SLOTS];
+    __shared__ int s_best;
     CtlCC* ctl = p.ctl;
-    const unsigned nblocks = gridDim.x;
+    int32_t* L = p.label;
     const unsigned lane = lane_id();
     const long long gtid = (long long)blockIdx.x * CC_T + threadIdx.x;
     const long long gthreads = (long long)gridDim.x * CC_T;
-    const long long gwarp = gtid >> 5, nwarps = gthreads >> 5;
     unsigned bar_target = 0;
+    int pass = 0, iters = 0;
 
-    // L_0 = identity, F_0 = vertices with an edge (phantom bits past n stay clear)
-    for (long long v = gtid; v < p.n; v += gthreads) p.label[v] = (int32_t)v;
-    for (long long w = gtid; w < p.W; w += gthreads) {
-        unsigned bits = ~__ldg(p.isolated + w);
-        if (w == p.W - 1 && (p.n & 31)) bits &= (1u << (p.n & 31)) - 1u;
-        p.F0[w] = bits;
-        p.F1[w] = 0u;
+    // every vertex points to its first neighbour if that is smaller
+    for (long long v = gtid; v < p.n; v += gthreads) {
+        const int b = __ldg(p.row_ptr + v), e = __ldg(p.row_ptr + v + 1);
+        int l = (int)v;
+        if (b < e) l = min(l, __ldg(p.col + b));
+        __stcg(L + v, l);
     }
-    // the fixed unit list of the big rows, for pull iterations
-    for (long long v0 = gwarp * 32; v0 < p.n; v0 += nwarps * 32) {  // warp-uniform
-        const long long v = v0 + lane;
-        const int deg = v < p.n ? __ldg(p.row_ptr + v + 1) - __ldg(p.row_ptr + v) : 0;
-        append_units_warp(p.B, &ctl->n_big, p.ucap, &ctl->bar.err, deg >= CC_CHUNK, (int)v, deg, CC_CHUNK);
+    if (p.m == 0) return;  // grid-uniform: every vertex is its own component
+    ++iters;
+    if (!grid_sync(&ctl->bar, gridDim.x, bar_target, p.timeout_ns)) return;
+    if (!cc_shortcut(p, bar_target, pass, iters)) return;
+    // the last neighbour of every row (a row's only entry is done if smaller)
+    for (long long v = gtid; v < p.n; v += gthreads) {
+        const int b = __ldg(p.row_ptr + v), e = __ldg(p.row_ptr + v + 1);
+        if (b == e) continue;
+        const int u = __ldg(p.col + e - 1);
+        if (e - b >= 2 || u > (int)v) cc_hook(L, cc_find(L, (int)v), u);
     }
-    if (gtid == 0) ctl->slot[0].changed = (unsigned long long)p.n;  // F_0: dense, so iteration 0 pulls
-    if (!grid_sync(&ctl->bar, nblocks, bar_target, p.timeout_ns)) return;
-    const long long n_big = (long long)min(__ldcg(&ctl->n_big), (unsigned long long)p.ucap);
+    ++iters;
+    if (!grid_sync(&ctl->bar, gridDim.x, bar_target, p.timeout_ns)) return;
+    if (!cc_shortcut(p, bar_target, pass, iters)) return;
 
-    int it = 0;
-    for (;; ++it) {
-        CountersCC* cur = &ctl->slot[it % 3];
-        CountersCC* nxt = &ctl->slot[(it + 1) % 3];
-        const unsigned long long* const csrc[2] = {&cur->changed, &cur->u_len};
-        unsigned long long cv[2];
-        cta_load_u64<2>(csrc, cv);
-        if (cv[0] == 0 && cv[1] == 0) break;
-        if (it >= p.max_iters) {
-            if (gtid == 0) atomicCAS(&ctl->bar.err, 0, (int)DEV_LEVELS);
-            break;
-        }
-        if (gtid == 0) {
-            CountersCC* z = &ctl->slot[(it + 2) % 3];
-            z->changed = 0;
-            z->u_len = 0;
-        }
-        uint32_t* f_cur = (it & 1) ? p.F1 : p.F0;
-        uint32_t* f_nxt = (it & 1) ? p.F0 : p.F1;
-        const int2* u_cur = (it & 1) ? p.U1 : p.U0;
-        int2* u_nxt = (it & 1) ? p.U0 : p.U1;
-        unsigned long long cnt = 0;
-        if (cv[0] * CC_PULL_DIV > (unsigned long long)p.n) {
-            cc_pull<CC_T>(p, f_cur, f_nxt, u_cur, (long long)min(cv[1], (unsigned long long)p.ucap), n_big, cnt);
-            cc_count(nxt, cnt, s_red);
-            if (!grid_sync(&ctl->bar, nblocks, bar_target, p.timeout_ns)) return;
-            cc_jump(p, f_nxt);
-            if (!grid_sync(&ctl->bar, nblocks, bar_target, p.timeout_ns)) return;
-            continue;
-        }
-
-        // chunk units of the previous iteration's big rows: a CTA per unit, an edge per thread
-        // (an overflow was recorded and its units dropped; never read past the list)
-        const long long nunits = (long long)min(cv[1], (unsigned long long)p.ucap);
-        for (long long u = blockIdx.x; u < nunits; u += gridDim.x) {
-            const int2 un = __ldcg(u_cur + u);
-            const int s = un.x;
-            const int ls = __ldcg(p.label + s);
-            const int b = __ldg(p.row_ptr + s) + un.y * CC_CHUNK;
-            const int e = min(__ldg(p.row_ptr + s + 1), b + CC_CHUNK);
-            const int j = b + (int)threadIdx.x;
-            if (j < e) cc_relax(p, f_nxt, ls, __ldg(p.col + j), cnt);
-        }
-
-        // the words of F_i, 32 of the dealing order loaded a step (one per lane);
-        // each non-empty word's rows flattened over the warp
-        const long long per = (p.W + nwarps - 1) / nwarps;
-        const long long iend = min((gwarp + 1) * per, (long long)p.W);
-        for (long long i0 = gwarp * per; i0 < iend; i0 += 32) {
-            const long long il = i0 + (long long)lane;
-            const long long wl = il < iend ? cc_word(p, il) : -1;
-            const unsigned fwl = wl >= 0 ? __ldcg(f_cur + wl) : 0u;
-            if (fwl) f_cur[wl] = 0u;  // the buffer holds F_{i+2} next
-            for (unsigned todo = __ballot_sync(0xffffffffu, fwl != 0); todo; todo &= todo - 1) {  // warp-uniform
-                const int src = __ffs(todo) - 1;
-                const long long w = __shfl_sync(0xffffffffu, wl, src);
-                const unsigned fw = __shfl_sync(0xffffffffu, fwl, src);
-                const bool act = (fw >> lane) & 1u;
-                const int s = (int)(w * 32 + lane);
-                int beg = 0, deg = 0, ls = 0;
-                if (act) {
-                    beg = __ldg(p.row_ptr + s);
-                    deg = __ldg(p.row_ptr + s + 1) - beg;
-                    ls = __ldcg(p.label + s);
-                }
-                const bool big = act && deg >= CC_CHUNK;
-                append_units_warp(u_nxt, &nxt->u_len, p.ucap, &p.ctl->bar.err, big, s, deg, CC_CHUNK);
-                const int fdeg = (act && !big) ? deg : 0;
-                int incl = fdeg;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int y = __shfl_up_sync(0xffffffffu, incl, o);
-                    if ((int)lane >= o) incl += y;
-                }
-                const int total = __shfl_sync(0xffffffffu, incl, 31);
-                const int excl = incl - fdeg;
-                for (int base = 0; base < total; base += 32) {
-                    const int idx = base + (int)lane;
-                    // owner: the last lane whose first entry is at or before idx
-                    int o = 0;
-#pragma unroll
-                    for (int st = 16; st > 0; st >>= 1) {
-                        const int ex = __shfl_sync(0xffffffffu, excl, (o + st) & 31);
-                        if (o + st < 32 && ex <= idx) o += st;
-                    }
-                    const int ob = __shfl_sync(0xffffffffu, beg, o);
-                    const int oex = __shfl_sync(0xffffffffu, excl, o);
-                    const int ol = __shfl_sync(0xffffffffu, ls, o);
-                    if (idx < total) cc_relax(p, f_nxt, ol, __ldg(p.col + ob + (idx - oex)), cnt);
-                }
+    // the label most sampled vertices carry; every CTA takes the same sample
+    // (labels do not change before the next barrier) and so the same label
+    for (int i = threadIdx.x; i < CC_SLOTS; i += CC_T) {
+        s_key[i] = -1;
+        s_cnt[i] = 0;
+    }
+    if (threadIdx.x == 0) s_best = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < CC_SAMPLES; i += CC_T) {
+        const unsigned long long h = (unsigned long long)(unsigned)i * 2654435761ull + 12345ull;
+        const int l = __ldcg(L + (long long)(h % (unsigned long long)p.n));
+        unsigned s = ((unsigned)l * 2654435761u) >> 21;  // 11 bits: CC_SLOTS
+        for (int tries = 0; tries < CC_SLOTS; ++tries, s = (s + 1) & (CC_SLOTS - 1)) {
+            const int old = atomicCAS(&s_key[s], -1, l);
+            if (old == -1 || old == l) {
+                atomicAdd(&s_cnt[s], 1);
+                break;
             }
         }
-
-        cc_count(nxt, cnt, s_red);
-        if (!grid_sync(&ctl->bar, nblocks, bar_target, p.timeout_ns)) return;
-        cc_jump(p, f_nxt);
-        if (!grid_sync(&ctl->bar, nblocks, bar_target, p.timeout_ns)) return;
     }
-    if (gtid == 0) ctl->iters = it;
+    __syncthreads();
+    for (int i = threadIdx.x; i < CC_SLOTS; i += CC_T) atomicMax(&s_best, s_cnt[i]);
+    __syncthreads();
+    const int best = s_best;
+    __syncthreads();
+    if (threadIdx.x == 0) s_best = INT32_MAX;
+    __syncthreads();
+    for (int i = threadIdx.x; i < CC_SLOTS; i += CC_T)
+        if (s_key[i] >= 0 && s_cnt[i] == best) atomicMin(&s_best, s_key[i]);
+    __syncthreads();
+    const int giant = s_best;
+    if (!grid_sync(&ctl->bar, gridDim.x, bar_target, p.timeout_ns)) return;
+
+    // the rows, but for their last entries, of every vertex outside that tree
+    // (the first entry has been hooked only if it was smaller): short rows by
+    // their lane, longer ones by the warp, the longest listed for the grid
+    for (long long v0 = gtid - lane; v0 < p.n; v0 += gthreads) {  // warp-uniform
+        const long long v = v0 + lane;
+        int b = 0, e = 0;
+        if (v < p.n && __ldcg(L + v) != giant) {
+            b = __ldg(p.row_ptr + v);
+            e = __ldg(p.row_ptr + v + 1) - 1;
+        }
+        const int len = e - b;
+        if (len >= CC_BIG_ROW - 1) {
+            const int at = atomicAdd(&ctl->n_big, 1);
+            if (at < p.big_cap) p.big[at] = (int)v;
+            else atomicCAS(&ctl->bar.err, 0, (int)DEV_OVERFLOW);  // cannot happen: rows sum to m
+        } else if (len > 0 && len <= CC_WARP_ROW) {
+            int a = cc_find(L, (int)v);
+            for (int j = b; j < e; ++j) {
+                const int u = __ldg(p.col + j);
+                if (__ldcg(L + u) != a) a = cc_hook(L, a, u);
+            }
+        }
+        unsigned wm = __ballot_sync(0xffffffffu, len > CC_WARP_ROW && len < CC_BIG_ROW - 1);
+        while (wm) {
+            const int l = __ffs(wm) - 1;
+            wm &= wm - 1;
+            const int bl = __shfl_sync(0xffffffffu, b, l), el = __shfl_sync(0xffffffffu, e, l);
+            int a = cc_find(L, (int)(v0 + l));
+            for (int j = bl + (int)lane; j < el; j += 32) {
+                const int u = __ldg(p.col + j);
+                if (__ldcg(L + u) != a) a = cc_hook(L, a, u);
+            }
+            __syncwarp();
+        }
+    }
+    ++iters;
+    if (!grid_sync(&ctl->bar, gridDim.x, bar_target, p.timeout_ns)) return;
+    const int nb = min(*(volatile int*)&ctl->n_big, p.big_cap);
+    for (int i = 0; i < nb; ++i) {
+        const int v = __ldcg(p.big + i);
+        const int b = __ldg(p.row_ptr + v), e = __ldg(p.row_ptr + v + 1) - 1;
+        if (b + gtid < e) {
+            int a = cc_find(L, v);
+            for (long long j = b + gtid; j < e; j += gthreads) {
+                const int u = __ldg(p.col + j);
+                if (__ldcg(L + u) != a) a = cc_hook(L, a, u);
+            }
+        }
+    }
+    if (nb > 0 && !grid_sync(&ctl->bar, gridDim.x, bar_target, p.timeout_ns)) return;  // grid-uniform
+    if (!cc_shortcut(p, bar_target, pass, iters)) return;
+    if (gtid == 0) ctl->iters = iters;
 }
-
-__global__ void cc_count_units_kernel(const int32_t* row_ptr, int32_t n, unsigned long long* out) {
-    unsigned long long s = 0;
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n; v += (long long)gridDim.x * blockDim.x) {
-        const int d = row_ptr[v + 1] - row_ptr[v];
-        if (d >= CC_CHUNK) s += (unsigned long long)((d + CC_CHUNK - 1) / CC_CHUNK);
-    }
-    s = warp_sum(s);
-    if ((threadIdx.x & 31) == 0 && s) atomicAdd(out, s);
-}
-
-struct StreamAllocs {
-    cudaStream_t st;
-    void* ptrs[12] = {};
-    int k = 0;
-    explicit StreamAllocs(cudaStream_t s) : st(s) {}
-    template <typename T>
-    bool alloc(T** p, size_t count) {
-        if (cudaMallocAsync((void**)p, std::max<size_t>(count, 1) * sizeof(T), st) != cudaSuccess) return false;
-        ptrs[k++] = *p;
-        return true;
-    }
-    ~StreamAllocs() {
-        for (int i = 0; i < k; ++i) cudaFreeAsync(ptrs[i], st);
-    }
-};
 
 }  // namespace
 
@@ -399,52 +272,52 @@ extern "C" bfs_status bfs_components(const bfs_graph* gc, int32_t* label, int32_
     std::lock_guard<std::mutex> guard(g->lock);
     cudaStream_t st = (cudaStream_t)cuda_stream;
     const int32_t n = g->n;
-    const int64_t W = div_up(n, 32);
     const bool host = !is_device_ptr(label);
 
-    StreamAllocs sa(st);
-    unsigned long long* d_units;
-    if (!sa.alloc(&d_units, 1)) {
+    // control block and list of long rows, kept with the graph: the call
+    // waits for its kernel under the graph's lock, so no two calls share it
+    // in time (an allocation from the stream-ordered pool here cost a call
+    // about as long as the kernel, since the pool gives memory back at every
+    // synchronisation)
+    const int32_t big_cap = g->deg_max >= CC_BIG_ROW ? (int32_t)(g->m / CC_BIG_ROW) + 1 : 0;
+    if (!g->cc_scratch &&
+        cudaMalloc(&g->cc_scratch, sizeof(CtlCC) + sizeof(int32_t) * (size_t)std::max(big_cap, 1)) != cudaSuccess) {
         cudaGetLastError();
+        g->cc_scratch = nullptr;
         return fail(BFS_ENOMEM, "components scratch");
     }
-    BFS_CUDA(cudaMemsetAsync(d_units, 0, 8, st));
-    cc_count_units_kernel<<<num_sms() * 8, 256, 0, st>>>(g->row_ptr, n, d_units);
-    unsigned long long units = 0;
-    BFS_CUDA(cudaMemcpyAsync(&units, d_units, 8, cudaMemcpyDeviceToHost, st));
-    BFS_CUDA(cudaStreamSynchronize(st));
-
-    ParamsCC p{};
-    p.n = n;
-    p.W = W;
-    p.row_ptr = g->row_ptr;
-    p.col = g->col;
-    p.isolated = g->isolated;
-    p.ucap = (int64_t)units + 1;
-    uint64_t K = 2654435761ull % (uint64_t)W;  // a multiplier coprime to W makes the dealing a permutation
-    if (K == 0) K = 1;
-    while (std::gcd(K, (uint64_t)W) != 1) ++K;
-    p.wmul = K;
-    p.timeout_ns = 2000000000ll;
-    p.max_iters = n + 1;
     int32_t* d_label = label;
-    if ((host && !sa.alloc(&d_label, (size_t)n)) || !sa.alloc(&p.F0, (size_t)W) || !sa.alloc(&p.F1, (size_t)W) ||
-        !sa.alloc(&p.U0, (size_t)p.ucap) || !sa.alloc(&p.U1, (size_t)p.ucap) || !sa.alloc(&p.B, (size_t)p.ucap) ||
-        !sa.alloc(&p.ctl, 1)) {
+    if (host && cudaMallocAsync(&d_label, (size_t)n * sizeof(int32_t), st) != cudaSuccess) {
         cudaGetLastError();
         return fail(BFS_ENOMEM, "components workspace for n=%d", n);
     }
+    ParamsCC p{};
+    p.n = n;
+    p.m = g->m;
+    p.row_ptr = g->row_ptr;
+    p.col = g->col;
     p.label = d_label;
-    BFS_CUDA(cudaMemsetAsync(p.ctl, 0, sizeof(CtlCC), st));
+    p.ctl = (CtlCC*)g->cc_scratch;
+    p.big = (int32_t*)(p.ctl + 1);
+    p.big_cap = big_cap;
+    p.timeout_ns = 2000000000ll;
     int per_sm = 0;
-    BFS_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cc_kernel, CC_T, 0));
-    if (per_sm < 1) return fail(BFS_ECUDA, "components kernel does not fit on an SM");
-    void* args[] = {(void*)&p};
-    BFS_CUDA(cudaLaunchCooperativeKernel((const void*)cc_kernel, dim3(per_sm * num_sms()), dim3(CC_T), args, 0, st));
     CtlCC h{};
-    BFS_CUDA(cudaMemcpyAsync(&h, p.ctl, sizeof(CtlCC), cudaMemcpyDeviceToHost, st));
-    if (host) BFS_CUDA(cudaMemcpyAsync(label, d_label, (size_t)n * 4, cudaMemcpyDeviceToHost, st));
-    BFS_CUDA(cudaStreamSynchronize(st));
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cc_kernel, CC_T, 0);
+    if (e == cudaSuccess) e = cudaMemsetAsync(p.ctl, 0, sizeof(CtlCC), st);
+    if (e == cudaSuccess) {
+        // no more CTAs than vertices to give a thread each: a small graph's
+        // barriers then count fewer arrivals
+        const int64_t want = std::max<int64_t>(1, div_up(n, CC_T));
+        const int blocks = (int)std::min<int64_t>(want, (int64_t)std::max(per_sm, 1) * num_sms());
+        void* args[] = {(void*)&p};
+        e = cudaLaunchCooperativeKernel((const void*)cc_kernel, dim3(blocks), dim3(CC_T), args, 0, st);
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, p.ctl, sizeof(CtlCC), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess && host) e = cudaMemcpyAsync(label, d_label, (size_t)n * 4, cudaMemcpyDeviceToHost, st);
+    if (host) cudaFreeAsync(d_label, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return cuda_fail(e, "components");
     if (h.bar.err) return device_error(h.bar.err, p.timeout_ns);
     if (iterations) *iterations = h.iters;
     return BFS_OK;

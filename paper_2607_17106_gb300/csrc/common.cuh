@@ -55,6 +55,7 @@ struct bfs_graph {
     int32_t deg_max = 0;
     double deg_mean = 0, deg_var = 0;
     int64_t n_big_units = 0;      // sizing of push chunk units, per chunk size (set on first run)
+    void* cc_scratch = nullptr;   // bfs_components: control block and row list (cc.cu), made on first use
     std::mutex lock;
     bfsgb::Workspace1* ws1 = nullptr;
     bfsgb::WorkspaceMS* wsms = nullptr;
