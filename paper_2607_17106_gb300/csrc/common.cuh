@@ -45,10 +45,12 @@ struct bfs_graph {
     int64_t m = 0;            // directed CSR entries
     int32_t symmetric = 0;
     int32_t device = 0;
+    void* rows = nullptr;         // the allocation that holds row_ptr, col, isolated and a directed graph's csc_*
+    int32_t* hub_col = nullptr;   // csc_col of a symmetric graph with BFS_PULL_HUBS_FIRST
     int32_t* row_ptr = nullptr;   // [n+1]
     int32_t* col = nullptr;       // [m]
     int32_t* csc_ptr = nullptr;   // [n+1], == row_ptr when symmetric
-    int32_t* csc_col = nullptr;   // [m],   == col when symmetric
+    int32_t* csc_col = nullptr;   // [m],   == col when symmetric (or hub_col)
     uint32_t* isolated = nullptr; // [W] bit v set iff deg(v) == 0 (out- and in-degree)
     int32_t* perm = nullptr;      // [n] new id of each input vertex (BFS_REORDER_RCM), else null
     int32_t n_isolated = 0;
