@@ -47,6 +47,11 @@ int msbfs_sticky_error(bfs_graph* g);  // msbfs.cu
 bfs_status run_graph_mode(bfs_graph* g, Workspace1* w, Params1& p, int32_t src, int32_t* depth, int32_t* parent,
                           const bfs_options& o, cudaStream_t st);  // bfs_graph.cu
 
+int ell_width(int32_t deg_max);  // bfs_small.cu
+int ell_cluster_size(int width);
+bool ell_prepare(const bfs_graph* g, Workspace1* w, cudaStream_t st);
+cudaError_t ell_launch(Params1 p, int width, int cl, cudaStream_t st);
+
 void free_ws1(Workspace1* w) {
     if (!w) return;
     cudaFree(w->P);
@@ -57,6 +62,7 @@ void free_ws1(Workspace1* w) {
     }
     cudaFree(w->E);
     cudaFree(w->cta_cnt);
+    cudaFree(w->ell);
     cudaFree(w->ctl);
     cudaFree(w->d_sticky);
     cudaFree(w->stage_depth);
@@ -553,18 +559,35 @@ static int small_levels_for(const bfs_graph* g, const bfs_options& o) {
     return small_cluster_size();
 }
 
+// The small levels by bfs_small.cu: maximum degree at most 8, and a direction
+// rule that needs only the level's counters.  Width of its rows, 0 for no.
+static int small_rows_for(const bfs_graph* g, const bfs_options& o) {
+    if (o.policy != BFS_POLICY_HEURISTIC && o.policy != BFS_POLICY_PUSH) return 0;
+    return ell_width(g->deg_max);
+}
+
 // The small-level launch pair of one search: the -1 rows stored by the copy
 // engines' memset (the cluster's few SMs would take long to store them),
 // the cluster launch, then the grid-wide launch that finishes the search.
 template <typename L>
-static cudaError_t run_small_pair(Params1 q, int cl, const L& launcher, cudaStream_t st) {
+static cudaError_t run_small_pair(const bfs_graph* g, Workspace1* w, const bfs_options& o, Params1 q, int cl,
+                                  const L& launcher, cudaStream_t st) {
+    const int width = small_rows_for(g, o);
+    int ell_cl = width ? ell_cluster_size(width) : 0;
+    if (ell_cl && !ell_prepare(g, w, st)) ell_cl = 0;
     cudaError_t e = cudaMemsetAsync(q.depth, 0xff, (size_t)q.n * sizeof(int32_t), st);
     if (!e && q.parent) e = cudaMemsetAsync(q.parent, 0xff, (size_t)q.n * sizeof(int32_t), st);
     q.do_init = 1;
     q.level_count = INT32_MAX / 2;
     q.small_ef_max = (int64_t)cl * SMALL_T;  // about one frontier edge a thread
     q.rows_filled = 1;
-    if (!e) e = launch_small(q, cl, st);
+    if (ell_cl) {
+        q.ell = w->ell;
+        if (!e) e = cudaMemcpyAsync(q.P, q.isolated, (size_t)q.W * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st);
+        if (!e) e = ell_launch(q, width, ell_cl, st);
+    } else if (!e) {
+        e = launch_small(q, cl, st);
+    }
     q.do_init = 0;
     q.small_ef_max = 0;
     q.rows_filled = 0;
@@ -797,7 +820,7 @@ bfs_status run_single(bfs_graph* g, int32_t src_value, int32_t* depth, int32_t* 
         if (const int cl = small_levels_for(g, o)) {
             // the small levels in one cluster, the rest grid-wide (a launch
             // that finds the search done returns at once)
-            BFS_CUDA(run_small_pair(p, cl, launcher, st));
+            BFS_CUDA(run_small_pair(g, w, o, p, cl, launcher, st));
         } else {
             BFS_CUDA(launch(p));
         }
@@ -861,7 +884,7 @@ bfs_status run_single_many(bfs_graph* g, const int32_t* src_host, int32_t k, int
             q.depth = depth + (int64_t)si * g->n;
             q.parent = parent ? parent + (int64_t)si * g->n : nullptr;
             BFS_CUDA(cudaMemsetAsync(w->ctl, 0, sizeof(Ctl1), st));
-            BFS_CUDA(run_small_pair(q, cl, launcher, st));
+            BFS_CUDA(run_small_pair(g, w, o, q, cl, launcher, st));
         }
         return BFS_OK;
     }

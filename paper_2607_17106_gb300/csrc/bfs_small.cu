@@ -1,0 +1,358 @@
+// bfs_small.cu -- the small push-queue levels of a search on a graph of low
+// degree (grids, road networks), run by one thread-block cluster.
+//
+// Such a search has thousands of levels of a few thousand vertices, and a
+// level costs a chain of dependent round trips whatever its size.  In the
+// general kernel the chain is: queue entry (L2), column (HBM), visited OR (L2)
+// with the new vertex's row bounds (HBM), queue reservation, store drain,
+// barrier -- 6.2 us a level on the relabelled 4096^2 grid.  Here it is one
+// memory round trip and the cluster's hardware barrier:
+//   - adjacency in rows of W = 4 or 8 entries (-1 for none), one aligned
+//     sector a vertex, built once per graph.  A candidate's row is loaded
+//     beside the OR that claims it, and the claimer puts it in the queue
+//     entry {vertex, parent, row}: the next level needs no load at all
+//     before its own ORs;
+//   - queues in shared memory.  The k-th claim of CTA c goes to CTA
+//     (c + k) mod CL, into the part of its queue that belongs to c, as a
+//     store through distributed shared memory: no reservation at the
+//     receiver, and every CTA expands the same share of the next frontier
+//     wherever the wavefront runs (a CTA that kept its own claims would keep
+//     its patch of it).  The claim counts are pushed to every CTA the same
+//     way, so that after the barrier all reads are local;
+//   - depth and parent of a vertex are stored when its entry is expanded, at
+//     the start of the next level, and are done long before its barrier.
+// The level that would not fit, or that is not a push-queue level, is handed
+// to the grid-wide kernel with the state that kernel continues from.
+#include "level.cuh"
+
+#include <algorithm>
+
+namespace bfsgb {
+
+namespace {
+
+constexpr int ELL_T = 1024;
+
+template <int W>
+struct EllCfg {
+    static constexpr int PITCH = W + 2;             // {vertex, parent, row}, 8-byte multiples
+    static constexpr int PART = W == 4 ? 256 : 160; // entries a CTA's queue holds from one sender
+    static constexpr int GROUPS = ELL_T / W;        // entries a CTA expands at a time, W threads each
+};
+
+template <int W>
+size_t ell_smem(int cl) {
+    return (size_t)2 * cl * EllCfg<W>::PART * EllCfg<W>::PITCH * sizeof(int32_t);
+}
+
+// Largest frontier a level may have: a CTA gets at most f / cl + cl of its
+// entries, claims at most W for each, and cl * PART claims fit.
+template <int W>
+int64_t ell_max_frontier(int cl) {
+    return (int64_t)cl * (cl * EllCfg<W>::PART / W - cl);
+}
+
+__device__ __forceinline__ unsigned cluster_rank() {
+    unsigned r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ unsigned map_shared(const void* p, unsigned rank) {
+    unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_cluster2(unsigned a, int x, int y) {
+    asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ void st_cluster(unsigned a, unsigned x) {
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(a), "r"(x) : "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ void ell_row(const int32_t* __restrict__ ell, int v, int (&a)[4]) {
+    const int4 x = __ldg(reinterpret_cast<const int4*>(ell) + v);
+    a[0] = x.x, a[1] = x.y, a[2] = x.z, a[3] = x.w;
+}
+__device__ __forceinline__ void ell_row(const int32_t* __restrict__ ell, int v, int (&a)[8]) {
+    const int4 x = __ldg(reinterpret_cast<const int4*>(ell) + 2ll * v), y = __ldg(reinterpret_cast<const int4*>(ell) + 2ll * v + 1);
+    a[0] = x.x, a[1] = x.y, a[2] = x.z, a[3] = x.w;
+    a[4] = y.x, a[5] = y.y, a[6] = y.z, a[7] = y.w;
+}
+
+// Claims of a CTA in one level, and their degree sum above them: at most
+// cl * PART claims of degree W, so neither field overflows.
+constexpr int CNT_BITS = 14;
+
+// Entries CTA d receives from a sender with `cnt` claims, (d - sender) mod cl = off.
+__device__ __forceinline__ int part_len(int cnt, int off, int cl) { return (cnt - off + cl - 1) / cl; }
+
+template <int W>
+__global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
+    using C = EllCfg<W>;
+    static_assert(16 * C::PART < (1 << CNT_BITS) && 16 * C::PART * W < (1 << (32 - CNT_BITS)), "packed counts");
+    extern __shared__ __align__(16) int32_t ell_q[];  // [2][cl][PART][PITCH]
+    __shared__ unsigned s_cnt[2][16];                 // packed claims of each CTA, by level parity
+    __shared__ unsigned s_mine[2];                    // this CTA's, being counted
+    const int cl = (int)gridDim.x, lg = __ffs(cl) - 1, rank = (int)cluster_rank();
+    const int lane = (int)lane_id();
+    const int grp = (int)threadIdx.x / W, j = (int)threadIdx.x % W;
+    const int per = C::GROUPS / cl;            // groups that expand the entries of one sender
+    const int from = grp / per, r = grp % per; // warp-uniform sender: per * W >= 32
+    Ctl1* ctl = p.ctl;
+
+    if (threadIdx.x < 32) {
+        const int s = p.src_value;
+        if (lane < 16) {
+            s_cnt[0][lane] = 0;
+            s_cnt[1][lane] = 0;
+        }
+        __syncwarp();
+        if (lane == 0) {
+            s_mine[0] = s_mine[1] = 0;
+            int row[W], deg = 0;
+            ell_row(p.ell, s, row);
+#pragma unroll
+            for (int k = 0; k < W; ++k) deg += row[k] >= 0;
+            s_cnt[0][0] = (unsigned)deg << CNT_BITS | 1u;  // F_0 as if CTA 0 had claimed it
+            if (rank == 0) {
+                int32_t* e = ell_q;
+                e[0] = s;
+                e[1] = s;
+#pragma unroll
+                for (int k = 0; k < W; ++k) e[2 + k] = row[k];
+                // P holds the vertices without an edge; the source, and the bits past n
+                atomicOr(p.P + (s >> 5), 1u << (s & 31));
+                if (p.n & 31) atomicOr(p.P + p.W - 1, ~((1u << (p.n & 31)) - 1u));
+            }
+        }
+    }
+    cluster_sync();
+
+    int level = 0;
+    long long m_u = p.m, f_prev = 0, f = 0, e_f = 0;
+    bool done = false;
+    for (;; ++level) {
+        const int par = level & 1;
+        const unsigned mine = lane < cl ? s_cnt[par][lane] : 0u;
+        f = (long long)__reduce_add_sync(0xffffffffu, mine & ((1u << CNT_BITS) - 1u));
+        e_f = (long long)__reduce_add_sync(0xffffffffu, mine >> CNT_BITS);
+        if (f == 0) {
+            if (rank == 0 && threadIdx.x == 0 && p.log && level < p.log_cap) {
+                bfs_level_record rec;
+                rec.level = level;
+                rec.dir = -1;
+                rec.f = rec.e_f = 0;
+                rec.m_u = m_u;
+                rec.t_ns = (int64_t)globaltimer_ns();
+                p.log[level] = rec;
+            }
+            done = true;
+            break;
+        }
+        if (level >= p.max_levels) {
+            if (rank == 0 && threadIdx.x == 0) atomicCAS(&ctl->bar.err, 0, (int)DEV_LEVELS);
+            done = true;
+            break;
+        }
+        const long long mu = m_u - e_f;
+        const int dir = p.policy == BFS_POLICY_PUSH ? push_kind(p, f)
+                                                    : heuristic_dir(p, f, e_f, mu, f_prev, BFS_DIR_PUSH_QUEUE);
+        if (dir != BFS_DIR_PUSH_QUEUE || f > p.small_ef_max) break;
+        m_u = mu;
+        if (rank == 0 && threadIdx.x == 0 && p.log && level < p.log_cap) {
+            bfs_level_record rec;
+            rec.level = level;
+            rec.dir = dir;
+            rec.f = f;
+            rec.e_f = e_f;
+            rec.m_u = m_u;
+            rec.t_ns = (int64_t)globaltimer_ns();
+            p.log[level] = rec;
+        }
+        const int len = part_len((int)(__shfl_sync(0xffffffffu, mine, from) & ((1u << CNT_BITS) - 1u)),
+                                 (rank - from) & (cl - 1), cl);
+        const int32_t* q = ell_q + ((size_t)par * cl + from) * C::PART * C::PITCH;
+        int32_t* qn = ell_q + ((size_t)(par ^ 1) * cl + rank) * C::PART * C::PITCH;  // this CTA's part, at any receiver
+        for (int i0 = 0; i0 < len; i0 += per) {  // warp-uniform
+            int u = -1, w = -1;
+            if (i0 + r < len) {
+                const int32_t* e = q + (i0 + r) * C::PITCH;
+                u = e[0];
+                w = e[2 + j];
+                if (j == 0) {
+                    p.depth[u] = level;
+                    if (p.parent) p.parent[u] = e[1];
+                }
+            }
+            int row[W];
+#pragma unroll
+            for (int k = 0; k < W; ++k) row[k] = -1;
+            bool won = false;
+            if (w >= 0) {
+                ell_row(p.ell, w, row);  // in flight beside the OR; wasted where it loses
+                const unsigned bit = 1u << (w & 31);
+                won = !(atomicOr(p.P + (w >> 5), bit) & bit);
+            }
+            const unsigned cm = __ballot_sync(0xffffffffu, won);
+            if (!cm) continue;
+            int deg = 0;
+#pragma unroll
+            for (int k = 0; k < W; ++k) deg += row[k] >= 0;
+            const unsigned es = __reduce_add_sync(0xffffffffu, won ? (unsigned)deg : 0u);
+            unsigned base = 0;
+            if (lane == 0) base = atomicAdd(&s_mine[par], es << CNT_BITS | (unsigned)__popc(cm));
+            base = __shfl_sync(0xffffffffu, base, 0) & ((1u << CNT_BITS) - 1u);
+            if (won) {
+                const int k = (int)base + __popc(cm & lanemask_lt());
+                const unsigned a = map_shared(qn + (k >> lg) * C::PITCH, (unsigned)((rank + k) & (cl - 1)));
+                st_cluster2(a, w, u);
+#pragma unroll
+                for (int t = 0; t < W; t += 2) st_cluster2(a + 8 + 4 * t, row[t], row[t + 1]);
+            }
+        }
+        __syncthreads();  // every claim of the CTA is counted
+        if (threadIdx.x < (unsigned)cl)
+            st_cluster(map_shared(&s_cnt[par ^ 1][rank], threadIdx.x), s_mine[par]);
+        if (threadIdx.x == 32) s_mine[par ^ 1] = 0;  // pushed a level ago, counts the next one
+        f_prev = f;
+        cluster_sync();
+    }
+    // The frontier F_level that was not expanded: depths and parents, and the
+    // queue entries of the grid-wide kernel.  Nothing is left of a finished one.
+    if (f > 0) {
+        const int par = level & 1;
+        const unsigned mine = lane < cl ? s_cnt[par][lane] & ((1u << CNT_BITS) - 1u) : 0u;
+        int before = 0;  // entries of the CTAs before this one
+        for (int d = 0; d < rank; ++d) {
+            const int x = lane < cl ? part_len((int)mine, (d - lane) & (cl - 1), cl) : 0;
+            before += (int)__reduce_add_sync(0xffffffffu, (unsigned)x);
+        }
+        int4* Q = par ? p.Q1 : p.Q0;
+        for (int c = 0; c < cl; ++c) {
+            const int len = part_len((int)__shfl_sync(0xffffffffu, mine, c), (rank - c) & (cl - 1), cl);
+            const int32_t* q = ell_q + ((size_t)par * cl + c) * C::PART * C::PITCH;
+            for (int i = (int)threadIdx.x; i < len; i += ELL_T) {
+                const int u = q[i * C::PITCH];
+                p.depth[u] = level;
+                if (p.parent) p.parent[u] = q[i * C::PITCH + 1];
+                Q[before + i] = make_int4(u, __ldg(p.row_ptr + u), __ldg(p.row_ptr + u + 1), 0);
+            }
+            before += len;
+        }
+    }
+    if (rank == 0 && threadIdx.x == 0) {
+        Counters* c = &ctl->slot[level % 3];  // the others are zero
+        c->q_len = (unsigned long long)f;
+        c->e_f = (unsigned long long)e_f;
+        ctl->next_level = level;
+        ctl->prev_dir = BFS_DIR_PUSH_QUEUE;
+        ctl->bm_valid = -1;
+        ctl->q_valid = level;
+        // the grid-wide kernel takes a level's e_f off itself, but for level 0's
+        ctl->m_u = level > 0 ? m_u : m_u - e_f;
+        ctl->f_prev = f_prev;
+        ctl->done = done ? 1 : 0;
+        const int e = ld_volatile_i32(&ctl->bar.err);
+        if (e) atomicCAS(p.sticky, 0, e);
+    }
+}
+
+// ell[v][k] = k-th neighbour of v, or -1
+__global__ void ell_build_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col, int32_t n, int w,
+                                 int32_t* __restrict__ ell) {
+    const int64_t total = (int64_t)n * w;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t v = i / w;
+        const int b = __ldg(row_ptr + v) + (int)(i % w);
+        ell[i] = b < __ldg(row_ptr + v + 1) ? __ldg(col + b) : -1;
+    }
+}
+
+template <int W>
+cudaLaunchConfig_t ell_config(int cl, cudaLaunchAttribute* attr, cudaStream_t st) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(cl);
+    cfg.blockDim = dim3(ELL_T);
+    cfg.dynamicSmemBytes = ell_smem<W>(cl);
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = cl;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cfg;
+}
+
+// CTAs of the cluster: 16 where the GPU can co-schedule them, else 8 (0: neither)
+template <int W>
+int ell_cluster() {
+    static int cached[64] = {};
+    const int d = device_id();
+    if (d < 0 || d >= 64) return 0;
+    if (cached[d]) return cached[d] > 0 ? cached[d] : 0;
+    int found = -1;
+    auto k = bfs_small_kernel<W>;
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ell_smem<W>(16)) == cudaSuccess) {
+        cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        for (int cl : {16, 8}) {
+            cudaLaunchAttribute attr[1];
+            cudaLaunchConfig_t cfg = ell_config<W>(cl, attr, nullptr);
+            int nc = 0;
+            if (cudaOccupancyMaxActiveClusters(&nc, k, &cfg) == cudaSuccess && nc >= 1) {
+                found = cl;
+                break;
+            }
+        }
+    }
+    cudaGetLastError();  // an unsupported size leaves a non-sticky error
+    cached[d] = found;
+    return found > 0 ? found : 0;
+}
+
+}  // namespace
+
+int ell_width(int32_t deg_max) { return deg_max <= 4 ? 4 : deg_max <= 8 ? 8 : 0; }
+
+// Rows of ell_width entries in w->ell, made once per workspace.  False: no
+// memory for them, or the stream is being captured (no allocation there); the
+// search then takes the general kernel.
+bool ell_prepare(const bfs_graph* g, Workspace1* w, cudaStream_t st) {
+    if (w->ell) return true;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return false;
+    }
+    const int width = ell_width(g->deg_max);
+    if (cudaMalloc(&w->ell, (size_t)g->n * width * sizeof(int32_t)) != cudaSuccess) {
+        cudaGetLastError();
+        w->ell = nullptr;
+        return false;
+    }
+    const int64_t blocks = std::min<int64_t>(div_up((int64_t)g->n * width, 256), (int64_t)num_sms() * 32);
+    ell_build_kernel<<<(unsigned)blocks, 256, 0, st>>>(g->row_ptr, g->col, g->n, width, w->ell);
+    return true;  // a failed launch shows at the search's own
+}
+
+int ell_cluster_size(int width) { return width == 4 ? ell_cluster<4>() : width == 8 ? ell_cluster<8>() : 0; }
+
+// The small levels of the search p describes; p.P holds the isolated
+// vertices, the outputs -1 and the control block zeros.
+cudaError_t ell_launch(Params1 p, int width, int cl, cudaStream_t st) {
+    cudaLaunchAttribute attr[1];
+    if (width == 4) {
+        p.small_ef_max = ell_max_frontier<4>(cl);
+        cudaLaunchConfig_t cfg = ell_config<4>(cl, attr, st);
+        return cudaLaunchKernelEx(&cfg, bfs_small_kernel<4>, p);
+    }
+    p.small_ef_max = ell_max_frontier<8>(cl);
+    cudaLaunchConfig_t cfg = ell_config<8>(cl, attr, st);
+    return cudaLaunchKernelEx(&cfg, bfs_small_kernel<8>, p);
+}
+
+}  // namespace bfsgb

@@ -54,6 +54,7 @@ struct Workspace1 {
     unsigned* cta_cnt = nullptr;  // frontier_sort: one count per CTA of the persistent launch
     int64_t ecap = 0;
     Ctl1* ctl = nullptr;
+    int32_t* ell = nullptr;  // rows of 4 or 8 neighbours (bfs_small.cu), made on first use
     int* d_sticky = nullptr;
     int32_t* stage_depth = nullptr;
     int32_t* stage_parent = nullptr;
@@ -82,6 +83,7 @@ struct Params1 {
     const int32_t* __restrict__ csc_ptr;
     const int32_t* __restrict__ csc_col;
     const uint32_t* __restrict__ isolated;
+    const int32_t* __restrict__ ell;  // bfs_small.cu
     uint32_t* P;
     uint32_t* F0;
     uint32_t* F1;
@@ -119,7 +121,7 @@ struct Params1 {
     // launch control
     int32_t do_init;
     int32_t level_count;  // levels to run in this launch (host loop: 1)
-    int64_t small_ef_max; // cluster launch: leave before a level with more frontier edges (or a pull)
+    int64_t small_ef_max; // cluster launch: leave before a level with more frontier edges (bfs_small.cu: vertices) or a pull
     int32_t rows_filled;  // the -1 of the depth and parent rows was stored before the launch
 };
 
