@@ -48,9 +48,9 @@ bfs_status run_graph_mode(bfs_graph* g, Workspace1* w, Params1& p, int32_t src, 
                           const bfs_options& o, cudaStream_t st);  // bfs_graph.cu
 
 int ell_width(int32_t deg_max);  // bfs_small.cu
-int ell_cluster_size(int width);
+int ell_cluster_size(const bfs_graph* g, int width);
 bool ell_prepare(const bfs_graph* g, Workspace1* w, cudaStream_t st);
-cudaError_t ell_launch(Params1 p, int width, int cl, cudaStream_t st);
+cudaError_t ell_launch(const bfs_graph* g, Params1 p, int width, int cl, cudaStream_t st);
 
 void free_ws1(Workspace1* w) {
     if (!w) return;
@@ -573,7 +573,7 @@ template <typename L>
 static cudaError_t run_small_pair(const bfs_graph* g, Workspace1* w, const bfs_options& o, Params1 q, int cl,
                                   const L& launcher, cudaStream_t st) {
     const int width = small_rows_for(g, o);
-    int ell_cl = width ? ell_cluster_size(width) : 0;
+    int ell_cl = width ? ell_cluster_size(g, width) : 0;
     if (ell_cl && !ell_prepare(g, w, st)) ell_cl = 0;
     cudaError_t e = cudaMemsetAsync(q.depth, 0xff, (size_t)q.n * sizeof(int32_t), st);
     if (!e && q.parent) e = cudaMemsetAsync(q.parent, 0xff, (size_t)q.n * sizeof(int32_t), st);
@@ -584,7 +584,7 @@ static cudaError_t run_small_pair(const bfs_graph* g, Workspace1* w, const bfs_o
     if (ell_cl) {
         q.ell = w->ell;
         if (!e) e = cudaMemcpyAsync(q.P, q.isolated, (size_t)q.W * sizeof(uint32_t), cudaMemcpyDeviceToDevice, st);
-        if (!e) e = ell_launch(q, width, ell_cl, st);
+        if (!e) e = ell_launch(g, q, width, ell_cl, st);
     } else if (!e) {
         e = launch_small(q, cl, st);
     }

@@ -21,6 +21,10 @@
 //     way, so that after the barrier all reads are local;
 //   - depth and parent of a vertex are stored when its entry is expanded, at
 //     the start of the next level, and are done long before its barrier.
+// A level takes 2.0 us up to 2 M cells (OR and row 0.7 us, cluster barrier 0.7,
+// append 0.3, counters 0.3) and 3.4 us on the 4096^2 grid, whose rows and outputs
+// (400 MB touched at random by one cluster) miss L2 and the TLB: a search
+// of that grid 41.7 -> 19.2 ms.
 // The level that would not fit, or that is not a push-queue level, is handed
 // to the grid-wide kernel with the state that kernel continues from.
 #include "level.cuh"
@@ -87,10 +91,12 @@ __device__ __forceinline__ void ell_row(const int32_t* __restrict__ ell, int v, 
 // cl * PART claims of degree W, so neither field overflows.
 constexpr int CNT_BITS = 14;
 
-// Entries CTA d receives from a sender with `cnt` claims, (d - sender) mod cl = off.
-__device__ __forceinline__ int part_len(int cnt, int off, int cl) { return (cnt - off + cl - 1) / cl; }
+// Entries CTA d receives from a sender with `cnt` claims, (d - sender) mod cl = off, cl = 1 << lg.
+__device__ __forceinline__ int part_len(int cnt, int off, int lg) { return (cnt - off + (1 << lg) - 1) >> lg; }
 
-template <int W>
+// SPEC: the rows of all candidates are loaded beside their ORs, not only the
+// claimed ones' after them.
+template <int W, bool SPEC>
 __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
     using C = EllCfg<W>;
     static_assert(16 * C::PART < (1 << CNT_BITS) && 16 * C::PART * W < (1 << (32 - CNT_BITS)), "packed counts");
@@ -132,14 +138,14 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
     }
     cluster_sync();
 
-    int level = 0;
-    long long m_u = p.m, f_prev = 0, f = 0, e_f = 0;
+    // the counters fit in 32 bits: a CSR has less than 2^31 entries
+    int level = 0, m_u = (int)p.m, f_prev = 0, f = 0, e_f = 0;
     bool done = false;
     for (;; ++level) {
         const int par = level & 1;
         const unsigned mine = lane < cl ? s_cnt[par][lane] : 0u;
-        f = (long long)__reduce_add_sync(0xffffffffu, mine & ((1u << CNT_BITS) - 1u));
-        e_f = (long long)__reduce_add_sync(0xffffffffu, mine >> CNT_BITS);
+        f = (int)__reduce_add_sync(0xffffffffu, mine & ((1u << CNT_BITS) - 1u));
+        e_f = (int)__reduce_add_sync(0xffffffffu, mine >> CNT_BITS);
         if (f == 0) {
             if (rank == 0 && threadIdx.x == 0 && p.log && level < p.log_cap) {
                 bfs_level_record rec;
@@ -158,15 +164,16 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
             done = true;
             break;
         }
-        const long long mu = m_u - e_f;
-        const int dir = p.policy == BFS_POLICY_PUSH ? push_kind(p, f)
-                                                    : heuristic_dir(p, f, e_f, mu, f_prev, BFS_DIR_PUSH_QUEUE);
-        if (dir != BFS_DIR_PUSH_QUEUE || f > p.small_ef_max) break;
+        // push_kind and heuristic_dir after a push level, in 32-bit integers
+        // (the 64-bit conversions took a tenth of the level)
+        const int mu = m_u - e_f;
+        const bool pull = p.policy != BFS_POLICY_PUSH && (float)e_f * p.alpha > (float)mu && f > f_prev;
+        if (pull || (float)f * p.gamma > (float)p.n || f > (int)p.small_ef_max) break;
         m_u = mu;
         if (rank == 0 && threadIdx.x == 0 && p.log && level < p.log_cap) {
             bfs_level_record rec;
             rec.level = level;
-            rec.dir = dir;
+            rec.dir = BFS_DIR_PUSH_QUEUE;
             rec.f = f;
             rec.e_f = e_f;
             rec.m_u = m_u;
@@ -174,18 +181,20 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
             p.log[level] = rec;
         }
         const int len = part_len((int)(__shfl_sync(0xffffffffu, mine, from) & ((1u << CNT_BITS) - 1u)),
-                                 (rank - from) & (cl - 1), cl);
+                                 (rank - from) & (cl - 1), lg);
         const int32_t* q = ell_q + ((size_t)par * cl + from) * C::PART * C::PITCH;
         int32_t* qn = ell_q + ((size_t)(par ^ 1) * cl + rank) * C::PART * C::PITCH;  // this CTA's part, at any receiver
         for (int i0 = 0; i0 < len; i0 += per) {  // warp-uniform
             int u = -1, w = -1;
             if (i0 + r < len) {
                 const int32_t* e = q + (i0 + r) * C::PITCH;
+                const int up = e[1];
                 u = e[0];
                 w = e[2 + j];
+                if (w == up) w = -1;  // the parent is visited
                 if (j == 0) {
                     p.depth[u] = level;
-                    if (p.parent) p.parent[u] = e[1];
+                    if (p.parent) p.parent[u] = up;
                 }
             }
             int row[W];
@@ -193,9 +202,10 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
             for (int k = 0; k < W; ++k) row[k] = -1;
             bool won = false;
             if (w >= 0) {
-                ell_row(p.ell, w, row);  // in flight beside the OR; wasted where it loses
+                if (SPEC) ell_row(p.ell, w, row);  // in flight beside the OR; wasted where it loses
                 const unsigned bit = 1u << (w & 31);
                 won = !(atomicOr(p.P + (w >> 5), bit) & bit);
+                if (!SPEC && won) ell_row(p.ell, w, row);
             }
             const unsigned cm = __ballot_sync(0xffffffffu, won);
             if (!cm) continue;
@@ -228,12 +238,12 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
         const unsigned mine = lane < cl ? s_cnt[par][lane] & ((1u << CNT_BITS) - 1u) : 0u;
         int before = 0;  // entries of the CTAs before this one
         for (int d = 0; d < rank; ++d) {
-            const int x = lane < cl ? part_len((int)mine, (d - lane) & (cl - 1), cl) : 0;
+            const int x = lane < cl ? part_len((int)mine, (d - lane) & (cl - 1), lg) : 0;
             before += (int)__reduce_add_sync(0xffffffffu, (unsigned)x);
         }
         int4* Q = par ? p.Q1 : p.Q0;
         for (int c = 0; c < cl; ++c) {
-            const int len = part_len((int)__shfl_sync(0xffffffffu, mine, c), (rank - c) & (cl - 1), cl);
+            const int len = part_len((int)__shfl_sync(0xffffffffu, mine, c), (rank - c) & (cl - 1), lg);
             const int32_t* q = ell_q + ((size_t)par * cl + c) * C::PART * C::PITCH;
             for (int i = (int)threadIdx.x; i < len; i += ELL_T) {
                 const int u = q[i * C::PITCH];
@@ -289,14 +299,14 @@ cudaLaunchConfig_t ell_config(int cl, cudaLaunchAttribute* attr, cudaStream_t st
 }
 
 // CTAs of the cluster: 16 where the GPU can co-schedule them, else 8 (0: neither)
-template <int W>
+template <int W, bool SPEC>
 int ell_cluster() {
     static int cached[64] = {};
     const int d = device_id();
     if (d < 0 || d >= 64) return 0;
     if (cached[d]) return cached[d] > 0 ? cached[d] : 0;
     int found = -1;
-    auto k = bfs_small_kernel<W>;
+    auto k = bfs_small_kernel<W, SPEC>;
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ell_smem<W>(16)) == cudaSuccess) {
         cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
         for (int cl : {16, 8}) {
@@ -339,20 +349,34 @@ bool ell_prepare(const bfs_graph* g, Workspace1* w, cudaStream_t st) {
     return true;  // a failed launch shows at the search's own
 }
 
-int ell_cluster_size(int width) { return width == 4 ? ell_cluster<4>() : width == 8 ? ell_cluster<8>() : 0; }
+// Rows are loaded with the candidates while they fit in L2 (126 MB): on a
+// 1000^2 grid 2.24 us a level against 2.32, on the 4096^2 grid (268 MB of rows, two
+// thirds of the loads for vertices visited before) 3.85 against 3.57, equal
+// at 2900^2 (134 MB).
+static bool ell_speculate(const bfs_graph* g, int width) {
+    return (int64_t)g->n * width * (int64_t)sizeof(int32_t) <= ((int64_t)128 << 20);
+}
+
+int ell_cluster_size(const bfs_graph* g, int width) {
+    const bool spec = ell_speculate(g, width);
+    if (width == 4) return spec ? ell_cluster<4, true>() : ell_cluster<4, false>();
+    if (width == 8) return spec ? ell_cluster<8, true>() : ell_cluster<8, false>();
+    return 0;
+}
 
 // The small levels of the search p describes; p.P holds the isolated
 // vertices, the outputs -1 and the control block zeros.
-cudaError_t ell_launch(Params1 p, int width, int cl, cudaStream_t st) {
+cudaError_t ell_launch(const bfs_graph* g, Params1 p, int width, int cl, cudaStream_t st) {
+    const bool spec = ell_speculate(g, width);
     cudaLaunchAttribute attr[1];
     if (width == 4) {
         p.small_ef_max = ell_max_frontier<4>(cl);
         cudaLaunchConfig_t cfg = ell_config<4>(cl, attr, st);
-        return cudaLaunchKernelEx(&cfg, bfs_small_kernel<4>, p);
+        return cudaLaunchKernelEx(&cfg, spec ? bfs_small_kernel<4, true> : bfs_small_kernel<4, false>, p);
     }
     p.small_ef_max = ell_max_frontier<8>(cl);
     cudaLaunchConfig_t cfg = ell_config<8>(cl, attr, st);
-    return cudaLaunchKernelEx(&cfg, bfs_small_kernel<8>, p);
+    return cudaLaunchKernelEx(&cfg, spec ? bfs_small_kernel<8, true> : bfs_small_kernel<8, false>, p);
 }
 
 }  // namespace bfsgb
