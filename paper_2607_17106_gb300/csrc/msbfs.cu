@@ -5,13 +5,17 @@
 // read of G.  With seen_i the lanes that reached v before level i and front_i
 // the lanes whose frontier holds v:
 //   push: for u with front_i[u] != 0, for v in N(u):
-//           new = front_i[u] & ~seen[v]; atomicOr(next[v], new)
+//           new = front_i[u] & ~atomicOr(seen[v], front_i[u]); atomicOr(next[v], new)
 //   pull: for v with missing = ~seen[v] != 0, OR front_i[u] over in-neighbours
 //           u in ascending order, stopping once every missing lane is found
 //   then front_{i+1} = next and seen |= next: the three-array identity
 //   F_{i+1} = P_{i+1} AND NOT P_i of the paper's variant 26.
 // The ANY reduction picks, per lane, the first u (push: the one whose OR set
 // the bit; pull: the lowest-index in-neighbour), which is written as parent.
+// A push claims in `seen` itself: a lane is then found once whatever buffer
+// F_{i+1} is in, and a level ends with one grid barrier.  (Claiming in next[]
+// and folding it into seen afterwards took a second barrier and a pass over
+// the new frontier a level.)
 //
 // One cooperative kernel runs all levels of all units of a launch: units are
 // independent searches (possibly over different graphs: bfs_run_mixed), and
@@ -51,13 +55,13 @@ struct CountersMS {
     unsigned long long lanes;  // OR of the frontier masks: lanes that can still find vertices
     unsigned long long done_e; // degree sum of the vertices that the level left seen by every live lane
     unsigned long long pull_next;  // pull level: cursor of the warps over the words of the vertex range
+    unsigned long long long_len;   // deferred long rows of the (pull) level this slot is current in
 };
 
 struct CtlMS {
     GridBarrier bar;
     CountersMS slot[3];
     int32_t levels;
-    unsigned long long long_len;  // deferred long rows of the current pull level
 };
 
 struct WorkspaceMS {
@@ -77,6 +81,7 @@ struct WorkspaceMS {
     unsigned long long* acc_long = nullptr;  // their lanes found so far
     uint64_t* hist = nullptr;            // frontier masks of levels 0 .. MS_HIST-1, [MS_HIST][ncap]
     int* hist_dirty = nullptr;           // device flag, see ParamsMS
+    uint32_t* full = nullptr;            // see ParamsMS
 };
 
 void free_wsms(WorkspaceMS* w) {
@@ -94,6 +99,7 @@ void free_wsms(WorkspaceMS* w) {
     cudaFree(w->acc_long);
     cudaFree(w->hist);
     cudaFree(w->hist_dirty);
+    cudaFree(w->full);
     cudaFreeHost(w->h_ctl);
     delete w;
 }
@@ -137,6 +143,7 @@ struct ParamsMS {
     uint64_t* hist;  // frontier masks of the first MS_HIST levels (zero between units)
     int64_t ncap;    // vertices per history level
     int* hist_dirty; // set while a launch runs; still set at the next launch if it ended early
+    uint32_t* full;  // bit v: v has no in-edge, or every lane has seen it (bits past n are set): no pull scans it
 };
 
 // Unit fields kept in registers / shared memory while a unit runs.
@@ -172,11 +179,34 @@ constexpr int MS_LONG_ITEMS = 4;  // entries a thread tests per long-row chunk
 constexpr int MS_PULL_R = BFS_MS_PULL_R;  // in-neighbours loaded per serial pull step
 constexpr int MS_COOP_U = 4;  // 32-entry groups a warp loads per step when it finishes a long row
 // Words a warp takes at a time in a pull level: one while many vertices
-// still miss live lanes (costly words: finest balance), eight once few do
-// (the takes of one word each then queue on the cursor's atomics).
-constexpr int MS_PULL_CHUNK_DENSE = 1, MS_PULL_CHUNK_SPARSE = 8;
+// still miss live lanes (costly words: finest balance).  Once few do, up to
+// 32, so that the takes don't queue on the cursor's atomics and most words are
+// passed over by their bits in `full`, but at least MS_PULL_TAKES takes a
+// warp: the words that are left may cost hundreds of microseconds each (with
+// 32 words a take on 2^14 vertices, 16 warps had them all: 97 -> 320 us).
+constexpr int MS_PULL_CHUNK = 32, MS_PULL_TAKES = 4;
+
+// A level's constants.  These and the unit's live in shared memory: at 64
+// registers a thread (two CTAs an SM) they were spilled, and the spills were
+// 170 million memory requests of an RMAT-22 batch.
+struct MsLevelConst {
+    int32_t level;
+    int pull_chunk;              // pull: words a warp takes at a time
+    uint64_t* f_next;
+    int32_t* a_next;
+    int2* u_next;
+    CountersMS* next;
+    uint64_t live;               // lanes with a non-empty frontier F_i
+    unsigned long long* cursor;  // pull: next word to take (zero when the level starts)
+    unsigned long long* long_len;  // pull: deferred long rows (zero when the level starts)
+    bool sparse;                 // pull: few vertices miss live lanes
+    bool write_depth;            // depths of F_{i+1} are written now (levels past the history)
+    bool clear_cur;              // push: F_i's masks are zeroed as they are read (levels past the history)
+};
 
 struct MsSmem {
+    UnitView g;
+    MsLevelConst lv;
     int32_t* depth[64];
     int32_t* parent[64];
     int off[MS_T + 1];
@@ -188,26 +218,21 @@ struct MsSmem {
     int32_t qbuf[(MS_T / 32) * MS_QBUF];
     float feat[BFS_MLP_IN];
     float mlp_out;
-    unsigned long long red[MS_T / 32];
+    unsigned long long red[4][MS_T / 32];  // a level's e_f, |F|, done_e and lanes, one share a warp
     unsigned long long base;
+    int qlen[MS_T / 32];
+    unsigned long long cnt[6];             // counters of the level about to start, read as the barrier opens
 };
 
+// What a thread gathers in a level.  Degree sums fit in 32 bits: a vertex is
+// counted once, and a CSR has less than 2^31 entries.
 struct MsLevel {
-    int32_t level;
-    uint64_t* f_next;
-    int32_t* a_next;
-    int2* u_next;
-    CountersMS* next;
-    unsigned long long ef;   // degree sum of F_{i+1} vertices (this thread's share)
-    unsigned long long cnt;  // |{v : F_{i+1}[v] != 0}| (pull levels, this thread's share)
+    const MsLevelConst& c;
+    unsigned ef;             // degree sum of F_{i+1} vertices (this thread's share)
+    unsigned cnt;            // |{v : F_{i+1}[v] != 0}| (pull levels, this thread's share)
+    unsigned done_e;         // degree sum of vertices now seen by every live lane (this thread's share)
     uint64_t lanes;          // OR of the F_{i+1} masks this thread wrote
-    uint64_t live;           // lanes with a non-empty frontier F_i
-    unsigned long long done_e;  // degree sum of vertices now seen by every live lane (this thread's share)
-    int32_t* qbuf;
     int qn;                  // staged appends (warp-uniform)
-    unsigned long long* cursor;  // pull: next word to take (zero when the level starts)
-    int pull_chunk;              // pull: words a warp takes at a time
-    bool write_depth;        // depths of F_{i+1} are written now (levels past the history)
 };
 
 __device__ __forceinline__ void write_lanes(MsSmem& sm, uint64_t bits, int v, int par, int d, bool write_depth) {
@@ -223,56 +248,90 @@ __device__ __forceinline__ void ms_units(const ParamsMS& p, int2* u_out, Counter
     append_units(u_out, &c->u_len, p.ucap, &p.ctl->bar.err, v, deg, p.chunk);
 }
 
-__device__ __forceinline__ void ms_flush(MsLevel& L) {
+__device__ __forceinline__ void ms_flush(MsLevel& L, MsSmem& sm) {
+    const int32_t* qbuf = sm.qbuf + (threadIdx.x >> 5) * MS_QBUF;
     if (L.qn == 0) return;
     unsigned lane = lane_id();
     unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(&L.next->a_len, (unsigned long long)L.qn);
+    if (lane == 0) base = atomicAdd(&L.c.next->a_len, (unsigned long long)L.qn);
     base = __shfl_sync(0xffffffffu, base, 0);
     __syncwarp();
-    for (int i = (int)lane; i < L.qn; i += 32) L.a_next[base + i] = L.qbuf[i];
+    for (int i = (int)lane; i < L.qn; i += 32) L.c.a_next[base + i] = qbuf[i];
     __syncwarp();
     L.qn = 0;
 }
 
 // v entered F_{i+1} (first OR into its mask this level): stage it for the
 // active list, add its degree, split big rows into chunk units.  Warp-uniform.
-__device__ __forceinline__ void ms_emit(const ParamsMS& p, MsLevel& L, bool first, int v, int deg) {
+__device__ __forceinline__ void ms_emit(const ParamsMS& p, MsLevel& L, MsSmem& sm, bool first, int v, int deg) {
     unsigned cm = __ballot_sync(0xffffffffu, first);
     if (!cm) return;
     int c = __popc(cm);
-    if (L.qn + c > MS_QBUF) ms_flush(L);
+    if (L.qn + c > MS_QBUF) ms_flush(L, sm);
     if (first) {
-        L.qbuf[L.qn + __popc(cm & lanemask_lt())] = v;
-        L.ef += (unsigned long long)deg;
-        if (deg >= p.chunk) ms_units(p, L.u_next, L.next, v, deg);
+        sm.qbuf[(threadIdx.x >> 5) * MS_QBUF + L.qn + __popc(cm & lanemask_lt())] = v;
+        L.ef += (unsigned)deg;
+        if (deg >= p.chunk) ms_units(p, L.c.u_next, L.c.next, v, deg);
     }
     L.qn += c;
 }
 
-// Push candidate u -> v with frontier lanes fu: the lanes of fu that v has
-// not seen are ORed into next[v]; the OR's old value names exactly one
-// claimer per (v, lane), which writes that lane's depth and parent.
-__device__ __forceinline__ void ms_candidate(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, bool has,
-                                             int v, int u, uint64_t fu) {
+// Push candidate u -> v with frontier lanes fu: the lanes of fu that v has not
+// seen are ORed into seen[v], whose old value names exactly one claimer per
+// (v, lane); the claimer enters them in F_{i+1}[v] and writes their parent
+// (and depth).  Returns true for the first entry into F_{i+1}[v], with v's
+// degree in deg.
+template <bool PAR>
+__device__ __forceinline__ bool ms_claim(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, bool has, int v,
+                                         int u, uint64_t fu, int& deg) {
     uint64_t bits = 0;
+    // an ordinary load: hubs are read by thousands of threads, which the L1 then
+    // serves; lanes only grow, so a stale word costs an OR at most
     if (has) bits = fu & ~((const unsigned long long*)p.seen)[v];
-    bool first = false;
-    int deg = 0;
-    if (bits) {
-        uint64_t old = atomicOr((unsigned long long*)L.f_next + v, (unsigned long long)bits);
-        uint64_t nb = bits & ~old;
-        first = (old == 0);
-        L.lanes |= nb;
-        if (nb) write_lanes(sm, nb, v, u, L.level + 1, L.write_depth);
-        if (first) deg = __ldg(g.row_ptr + v + 1) - __ldg(g.row_ptr + v);
-    }
-    ms_emit(p, L, first, v, deg);
+    if (!bits) return false;
+    const uint64_t old = atomicOr((unsigned long long*)p.seen + v, (unsigned long long)bits);
+    const uint64_t nb = bits & ~old, now = old | bits;
+    if (!nb) return false;
+    const uint64_t in = atomicOr((unsigned long long*)L.c.f_next + v, (unsigned long long)nb);
+    L.lanes |= nb;
+    if (PAR || L.c.write_depth) write_lanes(sm, nb, v, u, L.c.level + 1, L.c.write_depth);
+    const bool done = (now & L.c.live) == L.c.live && (old & L.c.live) != L.c.live;
+    if (in == 0 || done) deg = __ldg(g.row_ptr + v + 1) - __ldg(g.row_ptr + v);
+    if (done) L.done_e += (unsigned)deg;
+    if (now == g.lanes) atomicOr(p.full + (v >> 5), 1u << (v & 31));
+    return in == 0;
 }
 
+template <bool PAR>
+__device__ __forceinline__ void ms_candidate(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, bool has,
+                                             int v, int u, uint64_t fu) {
+    int deg = 0;
+    const bool first = ms_claim<PAR>(p, g, L, sm, has, v, u, fu, deg);
+    ms_emit(p, L, sm, first, v, deg);
+}
+
+// End of a push level: the warps' staged appends, with one atomic for the CTA
+// (one a warp queued thousands of them on the counter's sector).  Block-uniform.
 template <int T>
-__device__ void ms_push_tile(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, int u,
-                             const uint64_t* f_cur) {
+__device__ void ms_flush_all(MsLevel& L, MsSmem& sm) {
+    const int warp = (int)(threadIdx.x >> 5), lane = (int)lane_id();
+    if (lane == 0) sm.qlen[warp] = L.qn;
+    __syncthreads();
+    int before = 0, total = 0;
+    for (int w = 0; w < T / 32; ++w) {
+        const int x = sm.qlen[w];
+        before += w < warp ? x : 0;
+        total += x;
+    }
+    if (total == 0) return;
+    if (threadIdx.x == 0) sm.base = atomicAdd(&L.c.next->a_len, (unsigned long long)total);
+    __syncthreads();
+    for (int i = lane; i < L.qn; i += 32) L.c.a_next[sm.base + before + i] = sm.qbuf[warp * MS_QBUF + i];
+    L.qn = 0;
+}
+
+template <int T, bool PAR>
+__device__ void ms_push_tile(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, int u, uint64_t* f_cur) {
     static_assert(T <= MS_T, "tile arrays are sized for MS_T threads");
     unsigned lane = lane_id();
     int beg = 0, end = 0;
@@ -280,8 +339,9 @@ __device__ void ms_push_tile(const ParamsMS& p, const UnitView& g, MsLevel& L, M
     if (u >= 0) {
         beg = __ldg(g.row_ptr + u);
         end = __ldg(g.row_ptr + u + 1);
-        fu = ((const unsigned long long*)f_cur)[u];
+        fu = f_cur[u];
         if (end - beg >= p.chunk) end = beg;  // chunk units cover it
+        else if (L.c.clear_cur) f_cur[u] = 0;   // read once, by this thread
     }
     // medium rows: 32-edge segments taken in turn by every warp of the CTA
     const bool med = (end - beg) >= p.medium;
@@ -303,7 +363,7 @@ __device__ void ms_push_tile(const ParamsMS& p, const UnitView& g, MsLevel& L, M
             const int j = sm.beg[lo] + ((s - sm.off[lo]) << 5) + (int)lane;
             const bool has = j < sm.lim[lo];
             const int v = has ? __ldg(g.col + j) : 0;
-            ms_candidate(p, g, L, sm, has, v, sm.src[lo], sm.fmask[lo]);
+            ms_candidate<PAR>(p, g, L, sm, has, v, sm.src[lo], sm.fmask[lo]);
         }
     }
     if (med) end = beg;
@@ -330,16 +390,16 @@ __device__ void ms_push_tile(const ParamsMS& p, const UnitView& g, MsLevel& L, M
             sf = sm.fmask[lo];
             v = __ldg(g.col + sm.beg[lo] + (k - sm.off[lo]));
         }
-        ms_candidate(p, g, L, sm, has, v, su, sf);
+        ms_candidate<PAR>(p, g, L, sm, has, v, su, sf);
     }
     __syncthreads();
 }
 
 // Push level: items = chunk units of big rows, then CTA tiles of the active
 // list, dealt round-robin over the CTAs.
-template <int T>
+template <int T, bool PAR>
 __device__ void ms_push_level(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, const int32_t* a_cur,
-                              const int2* u_cur, const uint64_t* f_cur, long long a, long long nunits) {
+                              const int2* u_cur, uint64_t* f_cur, long long a, long long nunits) {
     long long per_tile = (a + gridDim.x - 1) / gridDim.x;
     per_tile = per_tile < 1 ? 1 : (per_tile > T ? T : per_tile);
     long long nitems = nunits + (a + per_tile - 1) / per_tile;
@@ -354,15 +414,15 @@ __device__ void ms_push_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
                 int j = base + threadIdx.x;
                 bool has = j < hi;
                 int v = has ? __ldg(g.col + j) : 0;
-                ms_candidate(p, g, L, sm, has, v, u, fu);
+                ms_candidate<PAR>(p, g, L, sm, has, v, u, fu);
             }
         } else {
             long long q = (it - nunits) * per_tile + threadIdx.x;
             int u = (threadIdx.x < per_tile && q < a) ? a_cur[q] : -1;
-            ms_push_tile<T>(p, g, L, sm, u, f_cur);
+            ms_push_tile<T, PAR>(p, g, L, sm, u, f_cur);
         }
     }
-    ms_flush(L);
+    ms_flush_all<T>(L, sm);
 }
 
 __device__ __forceinline__ uint64_t warp_or64(uint64_t x) {
@@ -385,31 +445,36 @@ __device__ __forceinline__ uint64_t warp_or64(uint64_t x) {
 constexpr size_t MS_PIDX_BYTES = (size_t)(MS_T / 32) * 64 * 32 * sizeof(unsigned short);
 extern __shared__ __align__(16) unsigned short ms_pidx_smem[];
 
+template <bool PAR>
 __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, const uint64_t* f_cur) {
     const unsigned lane = lane_id();
     unsigned short* pidx = ms_pidx_smem + (threadIdx.x >> 5) * (64 * 32);
-    const int dnext = L.level + 1;
-    const long long W = (g.n + 31) >> 5;
+    const int W = (g.n + 31) >> 5;
     const unsigned long long* F = (const unsigned long long*)f_cur;
-    // warps take L.pull_chunk words at a time from a level-wide cursor: the
+    // this thread's counters in the push tiles' arrays, not in registers
+    const int me = (int)threadIdx.x;
+    sm.beg[me] = sm.lim[me] = sm.src[me] = 0;  // degree sum, vertices, degree sum of the finished
+    sm.fmask[me] = 0;                          // lanes
+    // warps take pull_chunk words at a time from a level-wide cursor: the
     // cost of a word varies by orders of magnitude (hubs, early exits), and a
     // fixed deal left most warps waiting at the level barrier.  The next take
     // is requested when a chunk starts, so its round trip overlaps the work.
-    const unsigned long long chunk = (unsigned long long)L.pull_chunk;
-    unsigned long long take = 0;
-    if (lane == 0) take = atomicAdd(L.cursor, chunk);
+    unsigned take = 0;  // W < 2^26, and each warp passes it by one take at most
+    if (lane == 0) take = (unsigned)atomicAdd(L.c.cursor, (unsigned long long)L.c.pull_chunk);
     for (;;) {  // warp-uniform
-        const long long w0 = (long long)__shfl_sync(0xffffffffu, take, 0);
+        const int w0 = (int)__shfl_sync(0xffffffffu, take, 0);
         if (w0 >= W) break;
-        if (lane == 0) take = atomicAdd(L.cursor, chunk);
-        const long long w1 = min(w0 + (long long)chunk, W);
-        for (long long w = w0; w < w1; ++w) {
-        const long long v = w * 32 + lane;
+        if (lane == 0) take = (unsigned)atomicAdd(L.c.cursor, (unsigned long long)L.c.pull_chunk);
+        // the vertices that need no look: the chunk's words of `full`, one a
+        // lane (chunk <= 32), where few are open; on a dense level, whose
+        // words nearly all have work, the constant bitmap
+        const bool mine = (int)lane < min(L.c.pull_chunk, W - w0);
+        const unsigned fl = mine ? (L.c.sparse ? __ldcg(p.full + w0 + lane) : __ldg(g.isolated + w0 + lane)) : 0xffffffffu;
+        for (unsigned todo = __ballot_sync(0xffffffffu, fl != 0xffffffffu); todo; todo &= todo - 1) {  // warp-uniform
+        const int v = (w0 + __ffs(todo) - 1) * 32 + (int)lane;
         uint64_t miss = 0;
-        if (v < g.n) {
-            bool iso = (__ldg(g.isolated + w) >> lane) & 1u;
-            if (!iso) miss = L.live & ~((const unsigned long long*)p.seen)[v];
-        }
+        if (!((__shfl_sync(0xffffffffu, fl, __ffs(todo) - 1) >> lane) & 1u) && v < g.n)
+            miss = L.c.live & ~((const unsigned long long*)p.seen)[v];
         if (!__ballot_sync(0xffffffffu, miss != 0)) continue;
         int beg = 0, end = 0;
         if (miss) {
@@ -423,11 +488,11 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
         if (lm) {
             unsigned long long base = 0;
             const int leader = __ffs(lm) - 1;
-            if ((int)lane == leader) base = atomicAdd(&p.ctl->long_len, (unsigned long long)__popc(lm));
+            if ((int)lane == leader) base = atomicAdd(L.c.long_len, (unsigned long long)__popc(lm));
             base = __shfl_sync(0xffffffffu, base, leader);
             if (longrow) {
                 const unsigned long long r = base + __popc(lm & lanemask_lt());
-                p.longv[r] = (int)v;
+                p.longv[r] = v;
                 p.acc_long[r] = 0;
                 miss = 0;
                 end = beg;
@@ -450,7 +515,7 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
                 const uint64_t got = fm[r] & miss & ~acc;
                 if (got) {
                     acc |= got;
-                    uint64_t b = got;
+                    uint64_t b = PAR ? got : 0ull;
                     while (b) {
                         int lj = __ffsll((long long)b) - 1;
                         pidx[lj * 32 + lane] = (unsigned short)(j - beg);
@@ -484,18 +549,30 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
                     mine |= fu[q];
                 }
                 const uint64_t got = warp_or64(mine);
-                uint64_t gb = got;
-                while (gb) {  // warp-uniform: the first (lowest index) provider of each lane
-                    const int bj = __ffsll((long long)gb) - 1;
+                if (PAR && got) {  // warp-uniform
+                    // the first provider of each lane, in entry order: a
+                    // lane's bits that no entry before its own supplies (an
+                    // exclusive OR scan over each group of 32), recorded by
+                    // that lane; a ballot per bit and group took as long
+                    uint64_t before = 0;  // supplied by the groups before
 #pragma unroll
                     for (int q = 0; q < MS_COOP_U; ++q) {
-                        const unsigned who = __ballot_sync(0xffffffffu, (fu[q] >> bj) & 1ull);
-                        if (who) {
-                            if (lane == 0) pidx[bj * 32 + l] = (unsigned short)(b2 + q * 32 + __ffs(who) - 1 - bl);
-                            break;
+                        const uint64_t x = fu[q] & ~before;
+                        if (!__any_sync(0xffffffffu, x != 0)) continue;
+                        uint64_t s = x;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const uint64_t y = __shfl_up_sync(0xffffffffu, (unsigned long long)s, o);
+                            if ((int)lane >= o) s |= y;
+                        }
+                        const uint64_t ex = __shfl_up_sync(0xffffffffu, (unsigned long long)s, 1);
+                        uint64_t nb = lane ? x & ~ex : x;
+                        before |= __shfl_sync(0xffffffffu, (unsigned long long)s, 31);
+                        while (nb) {
+                            pidx[(__ffsll((long long)nb) - 1) * 32 + l] = (unsigned short)(b2 + q * 32 + (int)lane - bl);
+                            nb &= nb - 1;
                         }
                     }
-                    gb &= gb - 1;
                 }
                 al |= got;
             }
@@ -504,30 +581,46 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
         }
         // depths and parents of the word, lane-major: for each lane found
         // anywhere in the word, its row entries of the 32 vertices go out together
-        uint64_t all = warp_or64(acc);
+        uint64_t all = PAR || L.c.write_depth ? warp_or64(acc) : 0ull;
         __syncwarp();
+        // (four lanes' parent gathers in flight: RMAT-24 14.17 -> 13.47 ms, one at a
+        // time each lane's gather is a round trip of the word's chain)
         while (all) {  // warp-uniform
-            const int bj = __ffsll((long long)all) - 1;
-            if ((acc >> bj) & 1ull) {
-                if (L.write_depth) sm.depth[bj][v] = dnext;
-                int32_t* pp = sm.parent[bj];
-                if (pp) pp[v] = __ldg(g.csc_col + beg + pidx[bj * 32 + lane]);
+            int bj[4], par[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                bj[i] = all ? __ffsll((long long)all) - 1 : -1;
+                all &= all - 1;  // 0 stays 0
+                const bool f = bj[i] >= 0 && ((acc >> bj[i]) & 1ull);
+                if (!f) bj[i] = -1;
+                par[i] = PAR && f ? __ldg(g.csc_col + beg + pidx[bj[i] * 32 + lane]) : 0;
             }
-            all &= all - 1;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (bj[i] < 0) continue;
+                if (L.c.write_depth) sm.depth[bj[i]][v] = L.c.level + 1;
+                int32_t* pp = PAR ? sm.parent[bj[i]] : nullptr;
+                if (pp) pp[v] = par[i];
+            }
         }
         __syncwarp();
         if (acc) {
-            ((unsigned long long*)L.f_next)[v] = acc;
-            ((unsigned long long*)p.seen)[v] |= acc;
-            L.lanes |= acc;
-            L.cnt += 1;
-            const unsigned long long dv =
-                (unsigned long long)(g.symmetric ? (end - beg) : (__ldg(g.row_ptr + v + 1) - __ldg(g.row_ptr + v)));
-            L.ef += dv;
-            if (acc == miss) L.done_e += dv;  // no live lane misses v any more
+            ((unsigned long long*)L.c.f_next)[v] = acc;
+            const uint64_t now = ((const unsigned long long*)p.seen)[v] | acc;
+            ((unsigned long long*)p.seen)[v] = now;
+            if (now == g.lanes) atomicOr(p.full + (v >> 5), 1u << lane);
+            sm.fmask[me] |= acc;
+            sm.lim[me] += 1;
+            const unsigned dv = (unsigned)(g.symmetric ? (end - beg) : (__ldg(g.row_ptr + v + 1) - __ldg(g.row_ptr + v)));
+            sm.beg[me] += (int)dv;  // a degree sum below 2^31
+            if (acc == miss) sm.src[me] += (int)dv;  // no live lane misses v any more
         }
         }
     }
+    L.ef = (unsigned)sm.beg[me];
+    L.cnt = (unsigned)sm.lim[me];
+    L.done_e = (unsigned)sm.src[me];
+    L.lanes = sm.fmask[me];
 }
 
 // Long rows of a pull level: each is scanned by a whole CTA (rows dealt
@@ -535,7 +628,7 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
 // missing lane is found.  The CTA ORs the supplied lanes in shared memory and
 // keeps the first supplier of each lane as its parent; it owns the row, so
 // the accumulator and the parents are written with plain stores.
-template <int T>
+template <int T, bool PAR>
 __device__ void ms_long_rows(const ParamsMS& p, const UnitView& g, MsSmem& sm, const uint64_t* f_cur, uint64_t live,
                              long long nl) {
     __shared__ unsigned long long s_or;
@@ -559,7 +652,7 @@ __device__ void ms_long_rows(const ParamsMS& p, const UnitView& g, MsSmem& sm, c
                     const uint64_t got = F[u] & miss;
                     if (got) {
                         const uint64_t old = atomicOr(&s_or, (unsigned long long)got);
-                        uint64_t nb = got & ~old;
+                        uint64_t nb = PAR ? got & ~old : 0ull;
                         while (nb) {
                             const int b = __ffsll((long long)nb) - 1;
                             s_prov[b] = u;
@@ -572,7 +665,7 @@ __device__ void ms_long_rows(const ParamsMS& p, const UnitView& g, MsSmem& sm, c
         }
         const uint64_t acc = s_or;
         if (threadIdx.x == 0) p.acc_long[r] = acc;
-        if (threadIdx.x < 64 && ((acc >> threadIdx.x) & 1ull) && sm.parent[threadIdx.x])
+        if (PAR && threadIdx.x < 64 && ((acc >> threadIdx.x) & 1ull) && sm.parent[threadIdx.x])
             sm.parent[threadIdx.x][v] = s_prov[threadIdx.x];
         __syncthreads();
     }
@@ -603,6 +696,7 @@ __device__ void ms_long_finalize(const ParamsMS& p, const UnitView& g, MsSmem& s
         const unsigned long long dv = (unsigned long long)(__ldg(g.row_ptr + v + 1) - __ldg(g.row_ptr + v));
         ef += dv;
         if (((old | acc) & live) == live) done += dv;
+        if ((old | acc) == g.lanes) atomicOr(p.full + (v >> 5), 1u << (v & 31));
         ln |= acc;
     }
     cnt = warp_sum(cnt);
@@ -618,22 +712,45 @@ __device__ void ms_long_finalize(const ParamsMS& p, const UnitView& g, MsSmem& s
 }
 
 // Active list of F_i from its masks (after a pull level), with chunk units.
-template <int T>
-__device__ void ms_masks_to_list(const ParamsMS& p, const UnitView& g, MsSmem& sm, const uint64_t* f_cur,
-                                 int32_t* a_cur, int2* u_cur, CountersMS* cur) {
-    for (long long vb = (long long)blockIdx.x * T; vb < g.n; vb += (long long)gridDim.x * T) {
-        long long v = vb + threadIdx.x;
-        int flag = (v < g.n && ((const unsigned long long*)f_cur)[v] != 0) ? 1 : 0;
-        int total;
-        int off = block_exclusive_scan(flag, sm.scan_tmp, &total);
-        if (threadIdx.x == 0 && total) sm.base = atomicAdd(&cur->conv, (unsigned long long)total);
-        __syncthreads();
-        if (flag) {
-            a_cur[sm.base + off] = (int)v;
-            int deg = __ldg(g.row_ptr + v + 1) - __ldg(g.row_ptr + v);
-            if (deg >= p.chunk) ms_units(p, u_cur, cur, (int)v, deg);
+// A warp takes 8 x 32 masks at a time, all loaded before the first is looked
+// at, and appends with one atomic where it finds any: the frontier is sparse
+// here (after a pull level the next push has at most a few per cent of the
+// vertices), so reading the masks is the cost.  (A block scan per 512 masks took
+// 100 us for the 2^24 vertices of RMAT-24.)
+__device__ void ms_masks_to_list(const ParamsMS& p, const UnitView& g, const uint64_t* f_cur, int32_t* a_cur,
+                                 int2* u_cur, CountersMS* cur) {
+    constexpr int R = 8;
+    const unsigned lane = lane_id();
+    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+    const long long gwarp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    for (long long v0 = gwarp * (32 * R); v0 < g.n; v0 += nwarps * (32 * R)) {  // warp-uniform
+        unsigned long long m[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const long long v = v0 + r * 32 + lane;
+            m[r] = v < g.n ? __ldcg((const unsigned long long*)f_cur + v) : 0ull;
         }
-        __syncthreads();
+        unsigned b[R];
+        int total = 0;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            b[r] = __ballot_sync(0xffffffffu, m[r] != 0);
+            total += __popc(b[r]);
+        }
+        if (total == 0) continue;
+        unsigned long long at = 0;
+        if (lane == 0) at = atomicAdd(&cur->conv, (unsigned long long)total);
+        at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            if (m[r]) {
+                const int v = (int)(v0 + r * 32 + lane);
+                a_cur[at + __popc(b[r] & lanemask_lt())] = v;
+                const int deg = __ldg(g.row_ptr + v + 1) - __ldg(g.row_ptr + v);
+                if (deg >= p.chunk) ms_units(p, u_cur, cur, v, deg);
+            }
+            at += __popc(b[r]);
+        }
     }
 }
 
@@ -725,7 +842,7 @@ __device__ void ms_depth_pass(const ParamsMS& p, const UnitView& g, MsSmem& sm, 
     }
 }
 
-template <int T>
+template <int T, bool PAR>
 __device__ void msbfs_body(const ParamsMS& p) {
     __shared__ MsSmem sm;
     CtlMS* ctl = p.ctl;
@@ -744,21 +861,23 @@ __device__ void msbfs_body(const ParamsMS& p) {
     if (gtid == 0) *p.hist_dirty = 1;
     for (int ui = 0; ui < p.n_units; ++ui) {
         const MsUnit* U = p.units + ui;
-        UnitView g;
-        g.row_ptr = U->row_ptr;
-        g.col = U->col;
-        g.csc_ptr = U->csc_ptr;
-        g.csc_col = U->csc_col;
-        g.isolated = U->isolated;
-        g.m = U->m;
-        g.n = U->n;
-        g.k = U->k;
-        g.symmetric = U->symmetric;
-        g.lanes = (g.k >= 64) ? ~0ull : ((1ull << g.k) - 1);
+        UnitView& g = sm.g;
+        if (threadIdx.x == 0) {  // the last unit's readers have passed its closing barrier
+            g.row_ptr = U->row_ptr;
+            g.col = U->col;
+            g.csc_ptr = U->csc_ptr;
+            g.csc_col = U->csc_col;
+            g.isolated = U->isolated;
+            g.m = U->m;
+            g.n = U->n;
+            g.k = U->k;
+            g.symmetric = U->symmetric;
+            g.lanes = (U->k >= 64) ? ~0ull : ((1ull << U->k) - 1);
+        }
         int deg_max = U->deg_max;
         if (threadIdx.x < 64) {
-            sm.depth[threadIdx.x] = threadIdx.x < g.k ? U->depth[threadIdx.x] : nullptr;
-            sm.parent[threadIdx.x] = threadIdx.x < g.k ? U->parent[threadIdx.x] : nullptr;
+            sm.depth[threadIdx.x] = threadIdx.x < U->k ? U->depth[threadIdx.x] : nullptr;
+            sm.parent[threadIdx.x] = threadIdx.x < U->k ? U->parent[threadIdx.x] : nullptr;
         }
         __syncthreads();
         // init: masks, outputs (-1), counters
@@ -767,8 +886,13 @@ __device__ void msbfs_body(const ParamsMS& p) {
             p.F0[v] = 0;
             p.F1[v] = 0;
         }
+        for (long long w = gtid; w < (g.n + 31) >> 5; w += gthreads) {
+            unsigned bits = __ldg(g.isolated + w);
+            if (w * 32 + 32 > g.n) bits |= ~((1u << (g.n & 31)) - 1u);
+            p.full[w] = bits;
+        }
         // depths are written whole by ms_depth_pass; parents start at -1
-        for (int j = 0; j < g.k; ++j) {
+        for (int j = 0; PAR && j < g.k; ++j) {
             int32_t* pp = sm.parent[j];
             if (!pp) continue;
             for (long long v = gtid; v < g.n; v += gthreads) pp[v] = -1;
@@ -782,6 +906,7 @@ __device__ void msbfs_body(const ParamsMS& p) {
                 ctl->slot[s].lanes = 0;
                 ctl->slot[s].done_e = 0;
                 ctl->slot[s].pull_next = 0;
+                ctl->slot[s].long_len = 0;
             }
             ctl->slot[0].lanes = g.lanes;
         }
@@ -789,7 +914,8 @@ __device__ void msbfs_body(const ParamsMS& p) {
         if (blockIdx.x == 0 && threadIdx.x < (unsigned)g.k) {
             int j = threadIdx.x;
             int s = U->src[j];
-            atomicOr((unsigned long long*)p.seen + s, 1ull << j);
+            const unsigned long long was = atomicOr((unsigned long long*)p.seen + s, 1ull << j);
+            if ((was | 1ull << j) == g.lanes) atomicOr(p.full + (s >> 5), 1u << (s & 31));
             unsigned long long old = atomicOr((unsigned long long*)ms_front(p, 0) + s, 1ull << j);
             if (sm.parent[j]) sm.parent[j][s] = s;
             if (old == 0) {
@@ -805,13 +931,19 @@ __device__ void msbfs_body(const ParamsMS& p) {
         int prev_dir = BFS_DIR_PUSH_QUEUE;
         int unit_levels = 0;
         int list_valid = 0;  // level whose active list (and chunk units) exists
+        bool cnt_ok = false;     // sm.cnt holds the level's counters
         for (int level = 0;; ++level) {
             CountersMS* cur = &ctl->slot[level % 3];
             CountersMS* nxt = &ctl->slot[(level + 1) % 3];
-            const unsigned long long* const csrc[5] = {&cur->a_len, &cur->e_f, &cur->lanes, &cur->u_len,
-                                                       &cur->done_e};
             unsigned long long cv[5];
-            cta_load_u64<5>(csrc, cv);
+            if (cnt_ok) {
+#pragma unroll
+                for (int i = 0; i < 5; ++i) cv[i] = sm.cnt[i];
+            } else {
+                const unsigned long long* const csrc[5] = {&cur->a_len, &cur->e_f, &cur->lanes, &cur->u_len,
+                                                           &cur->done_e};
+                cta_load_u64<5>(csrc, cv);
+            }
             long long a = (long long)cv[0];
             long long e_f = (long long)cv[1];
             const uint64_t live = (uint64_t)cv[2];
@@ -842,7 +974,7 @@ __device__ void msbfs_body(const ParamsMS& p) {
             long long nunits = (long long)cv[3];
             if (dir != BFS_DIR_PULL && list_valid != level) {
                 // active list of a pull-made frontier (it appends the chunk units)
-                ms_masks_to_list<T>(p, g, sm, f_cur, a_cur, u_cur, cur);
+                ms_masks_to_list(p, g, f_cur, a_cur, u_cur, cur);
                 if (!grid_sync(&ctl->bar, nblocks, bar_target, p.timeout_ns)) return;
                 list_valid = level;
                 const unsigned long long* const usrc[1] = {&cur->u_len};
@@ -859,93 +991,89 @@ __device__ void msbfs_body(const ParamsMS& p) {
                 z->lanes = 0;
                 z->done_e = 0;
                 z->pull_next = 0;
+                z->long_len = 0;
             }
-            MsLevel L;
-            L.level = level;
-            L.f_next = ms_front(p, level + 1);
-            L.write_depth = level + 1 >= MS_HIST;
-            L.a_next = (level & 1) ? p.A0 : p.A1;
-            L.u_next = (level & 1) ? p.U0 : p.U1;
-            L.next = nxt;
-            L.ef = 0;
-            L.cnt = 0;
-            L.lanes = 0;
-            L.live = live;
-            L.done_e = 0;
-            L.qbuf = sm.qbuf + warp * MS_QBUF;
-            L.qn = 0;
-            L.cursor = &cur->pull_next;
-            // m_u: degree sum of the vertices some live lane has not seen
-            L.pull_chunk = 8 * m_u >= g.m ? MS_PULL_CHUNK_DENSE : MS_PULL_CHUNK_SPARSE;
-            if (dir == BFS_DIR_PULL) ms_pull_level(p, g, L, sm, f_cur);
-            else ms_push_level<T>(p, g, L, sm, a_cur, u_cur, f_cur, a, nunits);
+            if (threadIdx.x == 0) {  // its last readers have passed the level's barrier
+                MsLevelConst& c = sm.lv;
+                c.level = level;
+                c.f_next = ms_front(p, level + 1);
+                c.write_depth = level + 1 >= MS_HIST;
+                c.clear_cur = level >= MS_HIST;
+                c.a_next = (level & 1) ? p.A0 : p.A1;
+                c.u_next = (level & 1) ? p.U0 : p.U1;
+                c.next = nxt;
+                c.live = live;
+                c.cursor = &cur->pull_next;
+                c.long_len = &cur->long_len;
+                // m_u: degree sum of the vertices some live lane has not seen
+                c.sparse = 8 * m_u < g.m;
+                c.pull_chunk = 1;
+                if (c.sparse) {
+                    const int fair = ((g.n + 31) >> 5) / ((int)nblocks * (T / 32) * MS_PULL_TAKES);
+                    c.pull_chunk = min(max(fair, 1), MS_PULL_CHUNK);
+                }
+            }
+            __syncthreads();
+            MsLevel L{sm.lv, 0u, 0u, 0u, 0ull, 0};
+            const bool pull = dir == BFS_DIR_PULL;
+            if (pull) ms_pull_level<PAR>(p, g, L, sm, f_cur);
+            else ms_push_level<T, PAR>(p, g, L, sm, a_cur, u_cur, f_cur, a, nunits);
+            // the level's counters: a share a warp, one atomic each for the CTA
             const uint64_t ln = warp_or64(L.lanes);
-            if ((threadIdx.x & 31) == 0 && ln) atomicOr((unsigned long long*)&nxt->lanes, (unsigned long long)ln);
-            const unsigned long long dn = warp_sum(L.done_e);
-            if ((threadIdx.x & 31) == 0 && dn) atomicAdd(&nxt->done_e, dn);
-            unsigned long long ef = warp_sum(L.ef);
-            unsigned long long cn = warp_sum(L.cnt);
-            if ((threadIdx.x & 31) == 0) sm.red[warp] = ef;
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                unsigned long long t = 0;
-                for (int i = 0; i < T / 32; ++i) t += sm.red[i];
-                if (t) atomicAdd(&nxt->e_f, t);
+            const unsigned ef = __reduce_add_sync(0xffffffffu, L.ef), cn = __reduce_add_sync(0xffffffffu, L.cnt),
+                           dn = __reduce_add_sync(0xffffffffu, L.done_e);
+            if ((threadIdx.x & 31) == 0) {
+                sm.red[0][warp] = ef;
+                sm.red[1][warp] = cn;
+                sm.red[2][warp] = dn;
+                sm.red[3][warp] = ln;
             }
-            __syncthreads();
-            if (dir == BFS_DIR_PULL) {
-                if ((threadIdx.x & 31) == 0) sm.red[warp] = cn;
-                __syncthreads();
-                if (threadIdx.x == 0) {
-                    unsigned long long t = 0;
-                    for (int i = 0; i < T / 32; ++i) t += sm.red[i];
-                    if (t) atomicAdd(&nxt->a_len, t);
+            if (!pull) list_valid = level + 1;
+            // masks of F_i that were not zeroed as they were read, in a buffer F_{i+2} needs
+            const bool sweep = level >= MS_HIST && (pull || nunits > 0);
+            auto add = [&]() {
+                unsigned long long t[4] = {0, 0, 0, 0};
+                for (int i = 0; i < T / 32; ++i) {
+                    t[0] += sm.red[0][i];
+                    t[1] += sm.red[1][i];
+                    t[2] += sm.red[2][i];
+                    t[3] |= sm.red[3][i];
                 }
-            } else {
-                list_valid = level + 1;
+                if (t[0]) atomicAdd(&nxt->e_f, t[0]);
+                if (t[1]) atomicAdd(&nxt->a_len, t[1]);
+                if (t[2]) atomicAdd(&nxt->done_e, t[2]);
+                if (t[3]) atomicOr(&nxt->lanes, t[3]);
+            };
+            // read once the level is complete everywhere.  A CTA may be in the
+            // next level already: that changes neither these (its list
+            // conversion adds units, which are read again) nor this level's
+            // long_len, unless it is zero anyway or every CTA waits below
+            auto load = [&]() {
+                sm.cnt[0] = ld_cg_u64(&nxt->a_len);
+                sm.cnt[1] = ld_cg_u64(&nxt->e_f);
+                sm.cnt[2] = ld_cg_u64(&nxt->lanes);
+                sm.cnt[3] = ld_cg_u64(&nxt->u_len);
+                sm.cnt[4] = ld_cg_u64(&nxt->done_e);
+                sm.cnt[5] = ld_cg_u64(&cur->long_len);
+            };
+            if (!grid_sync(&ctl->bar, nblocks, bar_target, p.timeout_ns, add, load)) return;
+            const long long nl = pull ? (long long)sm.cnt[5] : 0;
+            if (nl > 0) {  // grid-uniform
+                ms_long_rows<T, PAR>(p, g, sm, f_cur, live, nl);
+                if (!grid_sync(&ctl->bar, nblocks, bar_target, p.timeout_ns)) return;
+                ms_long_finalize(p, g, sm, sm.lv.f_next, nl, level + 1, nxt, live, sm.lv.write_depth);
             }
-            if (!grid_sync(&ctl->bar, nblocks, bar_target, p.timeout_ns)) return;
-            long long nl = 0;
-            if (dir == BFS_DIR_PULL) {
-                const unsigned long long* const lsrc[1] = {&ctl->long_len};
-                unsigned long long lv[1];
-                cta_load_u64<1>(lsrc, lv);
-                nl = (long long)lv[0];
-                if (nl > 0) {
-                    ms_long_rows<T>(p, g, sm, f_cur, live, nl);
-                    if (!grid_sync(&ctl->bar, nblocks, bar_target, p.timeout_ns)) return;
-                    ms_long_finalize(p, g, sm, L.f_next, nl, level + 1, nxt, live, L.write_depth);
-                }
-            }
-            if (gtid == 0) ctl->long_len = 0;
-            // F_i is consumed: past the history its buffer is F_{i+2}'s, so
-            // clear its masks (history levels are kept for the depth pass);
-            // after a push level fold F_{i+1} into seen (a pull level already did)
-            if (level >= MS_HIST) {
-                if (list_valid >= level) {
-                    for (long long q = gtid; q < a; q += gthreads) f_cur[a_cur[q]] = 0;
-                } else {
+            if (sweep) {
+                if (pull) {
                     for (long long v = gtid; v < g.n; v += gthreads) f_cur[v] = 0;
+                } else {
+                    for (long long q = gtid; q < nunits; q += gthreads) f_cur[u_cur[q].x] = 0;
                 }
             }
-            if (dir != BFS_DIR_PULL) {
-                const unsigned long long* const asrc[1] = {&nxt->a_len};
-                unsigned long long av[1];
-                cta_load_u64<1>(asrc, av);
-                long long an = (long long)av[0];
-                unsigned long long done = 0;
-                for (long long q = gtid; q < an; q += gthreads) {
-                    const int v = L.a_next[q];
-                    const uint64_t old = p.seen[v];
-                    const uint64_t nw = old | ((const unsigned long long*)L.f_next)[v];
-                    p.seen[v] = nw;
-                    if ((nw & live) == live && (old & live) != live)
-                        done += (unsigned long long)(__ldg(g.row_ptr + v + 1) - __ldg(g.row_ptr + v));
-                }
-                done = warp_sum(done);
-                if ((threadIdx.x & 31) == 0 && done) atomicAdd(&nxt->done_e, done);
+            if (nl > 0 || sweep) {
+                if (!grid_sync(&ctl->bar, nblocks, bar_target, p.timeout_ns, NoArrivalWork(), load)) return;
             }
-            if (!grid_sync(&ctl->bar, nblocks, bar_target, p.timeout_ns)) return;
+            cnt_ok = true;
             a_prev = a;
             prev_dir = dir;
             ++total_levels;
@@ -961,9 +1089,10 @@ __device__ void msbfs_body(const ParamsMS& p) {
     }
 }
 
-template <int T>
+// PAR: some search of the launch wants its parents.
+template <int T, bool PAR>
 __global__ void __launch_bounds__(T, 2) msbfs_kernel(ParamsMS p) {
-    msbfs_body<T>(p);
+    msbfs_body<T, PAR>(p);
     if (threadIdx.x == 0) {
         int e = ld_volatile_i32(&p.ctl->bar.err);
         if (e) atomicCAS(p.sticky, 0, e);
@@ -1012,6 +1141,7 @@ static bfs_status alloc_wsms(int32_t ncap, int64_t ucap, int32_t chunk, int32_t 
     ok = ok && cudaMalloc(&w->acc_long, (size_t)ncap * 8) == cudaSuccess;
     ok = ok && cudaMalloc(&w->hist, (size_t)MS_HIST * ncap * 8) == cudaSuccess &&
          cudaMemset(w->hist, 0, (size_t)MS_HIST * ncap * 8) == cudaSuccess;
+    ok = ok && cudaMalloc(&w->full, (size_t)div_up(ncap, 32) * 4) == cudaSuccess;
     ok = ok && cudaMalloc(&w->hist_dirty, 4) == cudaSuccess && cudaMemset(w->hist_dirty, 0, 4) == cudaSuccess;
     ok = ok && cudaMallocHost(&w->h_ctl, sizeof(CtlMS)) == cudaSuccess;
     if (!ok) {
@@ -1023,10 +1153,10 @@ static bfs_status alloc_wsms(int32_t ncap, int64_t ucap, int32_t chunk, int32_t 
     return BFS_OK;
 }
 
-static int coop_blocks_ms(int blocks_per_sm) {
+static int coop_blocks_ms(const void* kernel, int blocks_per_sm) {
     int per_sm = 0;
-    cudaFuncSetAttribute(msbfs_kernel<MS_T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MS_PIDX_BYTES);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, msbfs_kernel<MS_T>, MS_T, MS_PIDX_BYTES);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MS_PIDX_BYTES);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, MS_T, MS_PIDX_BYTES);
     if (per_sm < 1) per_sm = 1;
     if (blocks_per_sm > 0) per_sm = std::min(per_sm, blocks_per_sm);
     return per_sm * num_sms();
@@ -1083,9 +1213,14 @@ static bfs_status launch_ms(WorkspaceMS* w, const std::vector<MsUnit>& units, co
     p.hist = w->hist;
     p.ncap = w->ncap;
     p.hist_dirty = w->hist_dirty;
-    int blocks = coop_blocks_ms(o.blocks_per_sm);
+    p.full = w->full;
+    bool par = false;
+    for (const MsUnit& u : units)
+        for (int j = 0; j < u.k; ++j) par |= u.parent[j] != nullptr;
+    const void* kernel = par ? (const void*)msbfs_kernel<MS_T, true> : (const void*)msbfs_kernel<MS_T, false>;
+    int blocks = coop_blocks_ms(kernel, o.blocks_per_sm);
     void* args[] = {(void*)&p};
-    BFS_CUDA(cudaLaunchCooperativeKernel((const void*)msbfs_kernel<MS_T>, dim3(blocks), dim3(MS_T), args, MS_PIDX_BYTES,
+    BFS_CUDA(cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(MS_T), args, MS_PIDX_BYTES,
                                          st));
     return BFS_OK;
 }
