@@ -1152,6 +1152,7 @@ extern "C" void bfs_free_graph(bfs_graph* g) {
     if (!g) return;
     free_ws1(g->ws1);
     free_wsms(g->wsms);
+    free_wsms(g->wsmix);
     cudaFree(g->rows);
     cudaFree(g->hub_col);
     cudaFree(g->perm);

@@ -56,11 +56,17 @@ struct bfs_graph {
     int32_t n_isolated = 0;
     int32_t deg_max = 0;
     double deg_mean = 0, deg_var = 0;
-    int64_t n_big_units = 0;      // sizing of push chunk units, per chunk size (set on first run)
     void* cc_scratch = nullptr;   // bfs_components: control block and row list (cc.cu), made on first use
     std::mutex lock;
     bfsgb::Workspace1* ws1 = nullptr;
     bfsgb::WorkspaceMS* wsms = nullptr;
+    // bfs_run_mixed: the workspace of the calls whose largest graph this is, and
+    // chunk units by chunk size, counted once (the graph does not change)
+    std::mutex mix_lock;
+    bfsgb::WorkspaceMS* wsmix = nullptr;
+    std::mutex units_lock;
+    int32_t units_chunk = 0;
+    int64_t units_count = 0;
 };
 
 namespace bfsgb {
