@@ -223,18 +223,18 @@ __global__ void __launch_bounds__(GT, 2) g_push(Params1 p) {
     L.next = nxt;
     L.ef = 0;
     L.cnt = 0;
-    L.qv = qs.qv + (threadIdx.x >> 5) * QBUF;
-    L.qb = qs.qb + (threadIdx.x >> 5) * QBUF;
-    L.qe = qs.qe + (threadIdx.x >> 5) * QBUF;
+    L.qs = qs.q + (threadIdx.x >> 5) * 3 * QBUF;
     L.qn = 0;
     L.qcap = p.n;
     L.err = &p.ctl->bar.err;
+    L.several = false;
+    L.append = false;
     L.precheck = push_precheck(h.m_u, p.m, h.e_f);
     const int4* q_cur = (level & 1) ? p.Q1 : p.Q0;
     const int2* u_cur = (level & 1) ? p.U1 : p.U0;
     const uint32_t* f_cur = (level & 1) ? p.F1 : p.F0;
     push_level<GT>(p, L, sm, DIR, q_cur, u_cur, f_cur, f, nunits, h.units_valid != 0);
-    unsigned long long ef = warp_sum(L.ef);
+    unsigned long long ef = (unsigned long long)__reduce_add_sync(0xffffffffu, L.ef);
     if ((threadIdx.x & 31) == 0) sm.red[threadIdx.x >> 5] = ef;
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -262,8 +262,8 @@ __global__ void __launch_bounds__(PULL_T) g_pull(Params1 p) {
     const uint32_t* f_cur = (level & 1) ? p.F1 : p.F0;
     uint32_t* f_next = (level & 1) ? p.F0 : p.F1;
     pull_level<true>(p, L, f_cur, f_next, s_pull[threadIdx.x >> 5]);
-    unsigned long long ef = warp_sum(L.ef);
-    unsigned long long cn = warp_sum(L.cnt);
+    unsigned long long ef = (unsigned long long)__reduce_add_sync(0xffffffffu, L.ef);
+    unsigned long long cn = (unsigned long long)__reduce_add_sync(0xffffffffu, L.cnt);
     if (lane_id() == 0) {
         s_ef[threadIdx.x >> 5] = ef;
         s_cn[threadIdx.x >> 5] = cn;

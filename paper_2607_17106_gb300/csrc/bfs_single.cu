@@ -94,19 +94,6 @@ constexpr size_t bfs1_dyn_smem() {
 }
 extern __shared__ __align__(16) unsigned char bfs1_dyn[];
 
-// a[0, len) = -1 by the whole grid: 16-byte stores from the first 16-byte
-// boundary, 4-byte stores for the head and the tail.  a is 4-byte aligned.
-__device__ __forceinline__ void fill_minus1(int32_t* a, long long len, long long gtid, long long gthreads) {
-    long long head = (long long)((16u - ((unsigned)(uintptr_t)a & 15u)) & 15u) >> 2;
-    if (head > len) head = len;
-    if (gtid < head) a[gtid] = -1;
-    const long long nv = (len - head) >> 2;
-    int4* const a4 = reinterpret_cast<int4*>(a + head);
-    for (long long i = gtid; i < nv; i += gthreads) a4[i] = make_int4(-1, -1, -1, -1);
-    const long long t0 = head + nv * 4;
-    if (gtid < len - t0) a[t0 + gtid] = -1;
-}
-
 // Address of `p` (this CTA's shared memory) in the cluster's CTA 0.
 template <typename X>
 __device__ __forceinline__ X* cluster_map_rank0(X* p) {
@@ -143,6 +130,14 @@ __device__ __forceinline__ bool level_sync(GridBarrier* b, unsigned nblocks, uns
     }
 }
 
+// A pull level that can find only few vertices (their degrees sum to at most
+// m_u) appends them to the next queue as it finds them: the push level that
+// follows (f < n / beta) then needs no pass over the bitmap and no barrier for
+// it (RMAT-22's sixth level 10.3 -> XX us).
+__device__ __forceinline__ bool pull_appends(const Params1& p, long long m_u) {
+    return p.symmetric && p.policy == BFS_POLICY_HEURISTIC && 256 * m_u <= (long long)p.n;
+}
+
 // SORT: the frontier-sort variants are compiled in (a separate instantiation,
 // so that the default kernel carries none of their registers).
 // CL: one thread-block cluster runs the small levels of one search (see
@@ -169,8 +164,9 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
     // One launch runs nsrc searches one after another (do_init), or continues
     // the search whose state the control block holds (host-loop drive).
     const int nsearch = p.do_init ? max(p.nsrc, 1) : 1;
+    // (32-bit counters: a CSR has less than 2^31 entries)
     int level = 0, prev_dir = BFS_DIR_PUSH_QUEUE, bm_valid = -1, q_valid = 0;
-    long long m_u = 0, f_prev = 0;
+    int m_u = 0, f_prev = 0;
     bool done = false;
     // counters of the level about to start (|F_i|, chunk units, e_f): set by
     // the init, or read by thread 0 right after the level barrier opens
@@ -195,9 +191,13 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
             if (w == p.W - 1 && (p.n & 31)) bits |= ~((1u << (p.n & 31)) - 1u);  // phantom vertices
             p.P[w] = bits;
         }
+        // (4-byte stores are as fast as 16-byte ones; setting only the entries a
+        // finished search had not reached, at its end, took longer: 64 searches
+        // of RMAT-22 8.47 ms against 8.22)
         if (!p.rows_filled) {
-            fill_minus1(depth, p.n, gtid, gthreads);
-            if (parent) fill_minus1(parent, p.n, gtid, gthreads);
+            for (long long v = gtid; v < p.n; v += gthreads) depth[v] = -1;
+            if (parent)
+                for (long long v = gtid; v < p.n; v += gthreads) parent[v] = -1;
         }
         __syncthreads();  // the CTA's warps have read s_cnt of the previous search's last level
         if (threadIdx.x == 0) {
@@ -242,7 +242,7 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
         prev_dir = BFS_DIR_PUSH_QUEUE;
         bm_valid = -1;
         q_valid = 0;
-        m_u = p.m - (long long)s_cnt[2];
+        m_u = (int)(p.m - (long long)s_cnt[2]);
         f_prev = 0;
         done = false;
         s_cnt_ok = true;
@@ -251,8 +251,8 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
         prev_dir = __ldcg(&ctl->prev_dir);
         bm_valid = __ldcg(&ctl->bm_valid);
         q_valid = __ldcg(&ctl->q_valid);
-        m_u = __ldcg(&ctl->m_u);
-        f_prev = __ldcg(&ctl->f_prev);
+        m_u = (int)__ldcg(&ctl->m_u);
+        f_prev = (int)__ldcg(&ctl->f_prev);
         done = __ldcg(&ctl->done) != 0;
     }
     const int level_end = level + p.level_count;
@@ -269,9 +269,8 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
             const unsigned long long* const csrc[3] = {&cur->q_len, &cur->u_len, &cur->e_f};
             cta_load_u64<3>(csrc, cv);
         }
-        long long f = (long long)cv[0];
-        long long nunits = (long long)cv[1];
-        long long e_f = (long long)cv[2];
+        const int f = (int)cv[0], e_f = (int)cv[2];
+        int nunits = (int)cv[1];
         if (f == 0) {
             // closing record: marks the end time of the last level
             if (gtid == 0 && p.log && level < p.log_cap) {
@@ -311,6 +310,22 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
             r.t_ns = (int64_t)globaltimer_ns();
             p.log[level] = r;
         }
+        if (m_u == 0 && p.symmetric && p.do_init) {
+            // no unvisited vertex has an edge: the level finds nothing, whatever
+            // its form (ER-22's last: 12,000 vertices, 125,000 edges, 10 us).
+            // Only in a launch that set the search up itself: one that continues
+            // from the control block has no barrier behind its threads' reads of
+            // it until it has run a level, and CTA 0 would write the state
+            // after this level over what other threads have still to read.
+            __syncthreads();  // every thread has read s_cnt
+            if (threadIdx.x < 3) s_cnt[threadIdx.x] = 0;
+            __syncthreads();
+            s_cnt_ok = true;
+            prev_dir = dir;
+            f_prev = f;
+            ++level;
+            continue;
+        }
         int2* u_cur = (level & 1) ? p.U1 : p.U0;
         uint32_t* f_cur = (level & 1) ? p.F1 : p.F0;
         uint32_t* f_nxt = (level & 1) ? p.F0 : p.F1;
@@ -337,7 +352,7 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
             const unsigned long long* const usrc[1] = {&cur->u_len};
             unsigned long long uv[1];
             cta_load_u64<1>(usrc, uv);
-            nunits = (long long)uv[0];
+            nunits = (int)uv[0];
             q_valid = level;
         } else if (dir == BFS_DIR_PUSH_QUEUE && q_valid != level) {
             // bitmap -> queue conversion of F_i (after pull levels)
@@ -346,7 +361,7 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
             const unsigned long long* const usrc[1] = {&cur->u_len};
             unsigned long long uv[1];
             cta_load_u64<1>(usrc, uv);
-            nunits = (long long)uv[0];
+            nunits = (int)uv[0];
             q_valid = level;
         }
         if (gtid == 0) {
@@ -366,12 +381,12 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
         L.next = nxt;
         L.ef = 0;
         L.cnt = 0;
-        L.qv = qs->qv + warp * QBUF;
-        L.qb = qs->qb + warp * QBUF;
-        L.qe = qs->qe + warp * QBUF;
+        L.qs = qs->q + warp * 3 * QBUF;
         L.qn = 0;
         L.qcap = p.n;
         L.err = &p.ctl->bar.err;
+        L.several = 2ll * e_f < p.m;
+        L.append = dir == BFS_DIR_PULL && pull_appends(p, m_u);
         L.precheck = push_precheck(m_u, p.m, e_f);
         if (dir == BFS_DIR_PULL) {
             pull_level_list<false, T>(p, L, f_cur, f_nxt, sm.list, reinterpret_cast<uint16_t*>(bfs1_dyn));
@@ -389,15 +404,14 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
         // e_f (and |F_{i+1}| for pull) of the next frontier: one atomic per
         // CTA, issued by thread 0 after the barrier's own __syncthreads and
         // before its arrival
-        const unsigned long long ef = warp_sum(L.ef);
-        const unsigned long long cn = warp_sum(L.cnt);
+        const unsigned ef = __reduce_add_sync(0xffffffffu, L.ef), cn = __reduce_add_sync(0xffffffffu, L.cnt);
         if ((threadIdx.x & 31) == 0) {
             sm.red[warp] = ef;
             sm.red2[warp] = cn;
         }
-        const bool pull_dir = dir == BFS_DIR_PULL;
+        const bool pull_dir = dir == BFS_DIR_PULL, count = pull_dir && !L.append;
         if (pull_dir) bm_valid = level + 1;
-        else q_valid = level + 1;
+        if (!pull_dir || L.append) q_valid = level + 1;
         prev_dir = dir;
         f_prev = f;
         const int done_level = level;
@@ -409,7 +423,7 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
                 tc += sm.red2[i];
             }
             if (te) atomicAdd(&nxt->e_f, te);
-            if (pull_dir && tc) atomicAdd(&nxt->q_len, tc);
+            if (count && tc) atomicAdd(&nxt->q_len, tc);
 #if BFS_LEVEL_PHASES
             if (p.log && done_level < p.log_cap / 2)
                 atomicMax((unsigned long long*)&p.log[p.log_cap / 2 + done_level].t_ns, (unsigned long long)globaltimer_ns());
@@ -590,7 +604,6 @@ static cudaError_t run_small_pair(const bfs_graph* g, Workspace1* w, const bfs_o
     }
     q.do_init = 0;
     q.small_ef_max = 0;
-    q.rows_filled = 0;
     if (!e) e = launcher(q, st);
     return e;
 }

@@ -122,7 +122,7 @@ struct Params1 {
     int32_t do_init;
     int32_t level_count;  // levels to run in this launch (host loop: 1)
     int64_t small_ef_max; // cluster launch: leave before a level with more frontier edges (bfs_small.cu: vertices) or a pull
-    int32_t rows_filled;  // the -1 of the depth and parent rows was stored before the launch
+    int32_t rows_filled;  // the -1 of the depth and parent rows was stored before the launch (else when the search ends)
 };
 
 // ------------------------------------------------------------- direction
@@ -185,7 +185,10 @@ __device__ inline int decide_dir(const Params1& p, int level, long long f, long 
 // rows make a few frontier words very hot, which the L1 then serves.
 
 // ------------------------------------------------------------ claiming
-constexpr int QBUF = 64;  // per-warp shared-memory staging of next-queue entries
+// Per-warp shared-memory staging of next-queue entries (64: every flush is an
+// atomic on the one queue counter; ER-22's widest push level has a million
+// appends, 15.26 -> 14.83 ms for 64 searches).
+constexpr int QBUF = 128;
 
 struct LevelCtx {
     int32_t level;          // i: discovered vertices get depth i+1
@@ -194,14 +197,15 @@ struct LevelCtx {
     int4* q_next;
     int2* u_next;
     Counters* next;         // counters of F_{i+1}
-    unsigned long long ef;  // this thread's share of e_f(F_{i+1})
-    unsigned long long cnt; // this thread's share of |F_{i+1}| (pull levels)
-    int32_t* qv;            // this warp's staging of next-queue entries (QBUF
-    int32_t* qb;            // each): vertex, row begin, row end
-    int32_t* qe;
+    unsigned ef;            // this thread's share of e_f(F_{i+1}): below 2^31 in all, as a CSR's entries are
+    unsigned cnt;           // this thread's share of |F_{i+1}| (pull levels)
+    int32_t* qs;            // this warp's staging of next-queue entries: QBUF
+                            // vertices, QBUF row begins, QBUF row ends
     int qn;                 // entries staged (warp-uniform)
-    long long qcap;         // capacity of q_next (n entries)
+    int qcap;               // capacity of q_next (n entries)
     int* err;               // device error word of the run
+    bool several;           // pull: test PULL_R2 entries a step (a scan is expected to need several)
+    bool append;            // pull: found vertices go to the next queue too
     bool precheck;          // push: read P before the OR (most targets already visited)
 };
 
@@ -232,7 +236,7 @@ __device__ __forceinline__ void flush_qbuf(LevelCtx& L) {
     // broken, record the overflow instead of writing past the buffer
     if (base + (unsigned long long)L.qn <= (unsigned long long)L.qcap) {
         for (int i = (int)lane; i < L.qn; i += 32) {
-            L.q_next[base + i] = make_int4(L.qv[i], L.qb[i], L.qe[i], 0);
+            L.q_next[base + i] = make_int4(L.qs[i], L.qs[QBUF + i], L.qs[2 * QBUF + i], 0);
         }
     } else if (lane == 0) {
         atomicCAS(L.err, 0, (int)DEV_OVERFLOW);
@@ -262,12 +266,12 @@ __device__ __forceinline__ void emit(const Params1& p, LevelCtx& L, bool claimed
     const int deg = re - rb;
     if (claimed) {
         const int slot = L.qn + __popc(cm & lanemask_lt());
-        L.qv[slot] = v;
-        L.qb[slot] = rb;
-        L.qe[slot] = re;
+        L.qs[slot] = v;
+        L.qs[QBUF + slot] = rb;
+        L.qs[2 * QBUF + slot] = re;
         L.depth[v] = L.level + 1;
         if (L.parent) L.parent[v] = u;
-        L.ef += (unsigned long long)deg;
+        L.ef += (unsigned)deg;
     }
     L.qn += c;
     emit_units_warp(p, L.u_next, L.next, claimed && deg >= p.chunk, v, deg);
@@ -321,7 +325,7 @@ __device__ __forceinline__ void flush_pairs(const Params1& p, LevelCtx& L) {
     base = __shfl_sync(0xffffffffu, base, 0);
     __syncwarp();
     if (base + (unsigned long long)L.qn <= (unsigned long long)p.ecap) {
-        for (int i = (int)lane; i < L.qn; i += 32) p.E[base + i] = make_int2(L.qv[i], L.qb[i]);
+        for (int i = (int)lane; i < L.qn; i += 32) p.E[base + i] = make_int2(L.qs[i], L.qs[QBUF + i]);
     } else if (lane == 0) {
         atomicCAS(&p.ctl->bar.err, 0, (int)DEV_OVERFLOW);
     }
@@ -341,7 +345,7 @@ __device__ __forceinline__ void flush_push(const Params1& p, LevelCtx& L) {
 // every pair (BFS_PUSH_FILTER, Variants 13/14: advance without the predicate),
 // or those whose v is not yet set in P (BFS_PUSH_FILTER_PREDICATED, Variants
 // 20/23: the visited test in the advance, the visited update in the filter).
-// The warp's queue staging holds the pairs (target in qv, source in qb).
+// The warp's queue staging holds the pairs (targets, then sources).
 // Warp-uniform.
 __device__ __forceinline__ void push_candidate(const Params1& p, LevelCtx& L, bool has, int v, int u) {
     if (p.push_filter == BFS_PUSH_FUSED) {
@@ -356,8 +360,8 @@ __device__ __forceinline__ void push_candidate(const Params1& p, LevelCtx& L, bo
     if (L.qn + c > QBUF) flush_pairs(p, L);
     if (want) {
         const int slot = L.qn + __popc(cm & lanemask_lt());
-        L.qv[slot] = v;
-        L.qb[slot] = u;
+        L.qs[slot] = v;
+        L.qs[QBUF + slot] = u;
     }
     L.qn += c;
 }
@@ -398,9 +402,7 @@ struct PullListSmem {
 // The warps' staging of next-queue entries in push levels (QBUF each).
 template <int T>
 struct QueueStage {
-    int32_t qv[(T / 32) * QBUF];
-    int32_t qb[(T / 32) * QBUF];
-    int32_t qe[(T / 32) * QBUF];
+    int32_t q[(T / 32) * 3 * QBUF];
 };
 
 // Shared memory of a CTA running level kernels.  Push levels use the tile
@@ -744,7 +746,7 @@ __device__ __forceinline__ void pull_words_scan(const Params1& p, LevelCtx& L, c
             const long long v = w * 32 + lane;
             L.depth[v] = dnext;
             if (L.parent) L.parent[v] = par[k];
-            L.ef += (unsigned long long)(p.symmetric ? (end[k] - beg[k])
+            L.ef += (unsigned)(p.symmetric ? (end[k] - beg[k])
                                                      : (__ldg(p.row_ptr + v + 1) - __ldg(p.row_ptr + v)));
             L.cnt += 1;
         }
@@ -821,7 +823,7 @@ __device__ __forceinline__ void pull_found(const Params1& p, LevelCtx& L, unsign
     atomicOr(nb + slot, 1u << (v & 31));
     L.depth[v] = L.level + 1;
     if (L.parent) L.parent[v] = u;
-    L.ef += (unsigned long long)(p.symmetric ? (e - b0) : (__ldg(p.row_ptr + v + 1) - __ldg(p.row_ptr + v)));
+    L.ef += (unsigned)(p.symmetric ? (e - b0) : (__ldg(p.row_ptr + v + 1) - __ldg(p.row_ptr + v)));
     L.cnt += 1;
 }
 
@@ -1046,12 +1048,33 @@ __device__ __forceinline__ void pull_level(const Params1& p, LevelCtx& L, const 
 // measured slower on RMAT, ER and BA).
 constexpr int PULL_LPI = 2;
 
+// Entries tested a step on levels whose frontier holds less than half of the
+// edges, so that most scans take more than one (ER-22, 64 searches: one entry
+// 14.83 ms, two 14.38, three 14.3, four 14.6; RMAT-22 8.67, 8.51, 8.53, 8.67).
+constexpr int PULL_R2 = 2;
+
+// Next-queue entries of the vertices a pull level found (symmetric graphs: the
+// in-row bounds are the row's).  Warp-uniform.
+__device__ __forceinline__ void append_found(const Params1& p, LevelCtx& L, bool found, int v, int beg, int end) {
+    const unsigned m = __ballot_sync(0xffffffffu, found);
+    if (!m) return;
+    unsigned long long base = 0;
+    if (lane_id() == 0) base = atomicAdd(&L.next->q_len, (unsigned long long)__popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (base + (unsigned long long)__popc(m) > (unsigned long long)L.qcap) {
+        if (lane_id() == 0) atomicCAS(L.err, 0, (int)DEV_OVERFLOW);
+    } else if (found) {
+        L.q_next[base + __popc(m & lanemask_lt())] = make_int4(v, beg, end, 0);
+    }
+    emit_units_warp(p, L.u_next, L.next, found && end - beg >= p.chunk, v, end - beg);
+}
+
 // Scans of up to PULL_LPI listed vertices per lane (v < 0: none), as in
 // pull_words_scan: ascending in-neighbours, the first one in F_i is the
 // parent; rows still open after `serial` entries are finished by the whole
 // warp, 4 x 32 entries a step.  Found vertices set their bit in the slot's
 // shared-memory word nb[sl].  Warp-uniform.
-template <bool NC>
+template <bool NC, bool SEVERAL>
 __device__ __forceinline__ void pull_list_scan(const Params1& p, LevelCtx& L, unsigned* nb, const uint32_t* f_cur,
                                                const int (&v)[PULL_LPI], const int (&sl)[PULL_LPI], int serial) {
     const unsigned lane = lane_id();
@@ -1065,6 +1088,39 @@ __device__ __forceinline__ void pull_list_scan(const Params1& p, LevelCtx& L, un
         par[q] = -1;
         found[q] = false;
     }
+    if (SEVERAL && L.several) {
+        constexpr int R = PULL_R2;
+        for (int step = 0; step < serial; step += R) {
+            int u[PULL_LPI][R];
+            unsigned fw[PULL_LPI][R];
+            bool live = false;
+#pragma unroll
+            for (int q = 0; q < PULL_LPI; ++q) {
+                const bool lk = !found[q] && j[q] < end[q];
+                live |= lk;
+#pragma unroll
+                for (int r = 0; r < R; ++r) u[q][r] = (lk && j[q] + r < end[q]) ? __ldg(p.csc_col + j[q] + r) : -1;
+            }
+            if (!live) break;
+#pragma unroll
+            for (int q = 0; q < PULL_LPI; ++q)
+#pragma unroll
+                for (int r = 0; r < R; ++r) fw[q][r] = u[q][r] >= 0 ? ld_word<NC>(f_cur, u[q][r] >> 5) : 0u;
+#pragma unroll
+            for (int q = 0; q < PULL_LPI; ++q) {
+                if (u[q][0] < 0) continue;
+                int adv = R;
+#pragma unroll
+                for (int r = R - 1; r >= 0; --r)
+                    if (u[q][r] >= 0 && ((fw[q][r] >> (u[q][r] & 31)) & 1u)) {
+                        adv = r;
+                        par[q] = u[q][r];
+                    }
+                found[q] = adv < R;
+                j[q] += adv;
+            }
+        }
+    } else {
     // software-pipelined scan: each step tests the current entry's F_i word
     // and loads the next entry, so a step costs one memory round trip (two
     // or four entries a step measured no faster)
@@ -1094,6 +1150,7 @@ __device__ __forceinline__ void pull_list_scan(const Params1& p, LevelCtx& L, un
                 u[q] = un[q];
             }
         }
+    }
     }
 #pragma unroll
     for (int q = 0; q < PULL_LPI; ++q) {
@@ -1125,11 +1182,12 @@ __device__ __forceinline__ void pull_list_scan(const Params1& p, LevelCtx& L, un
             }
             rm &= rm - 1;
         }
+        if (L.append) append_found(p, L, found[q], v[q], beg[q], end[q]);
         if (found[q]) {
             atomicOr(nb + sl[q], 1u << (v[q] & 31));
             L.depth[v[q]] = L.level + 1;
             if (L.parent) L.parent[v[q]] = par[q];
-            L.ef += (unsigned long long)(p.symmetric ? (end[q] - beg[q])
+            L.ef += (unsigned)(p.symmetric ? (end[q] - beg[q])
                                                      : (__ldg(p.row_ptr + v[q] + 1) - __ldg(p.row_ptr + v[q])));
             L.cnt += 1;
         }
@@ -1214,7 +1272,8 @@ __device__ void pull_level_list(const Params1& p, LevelCtx& L, const uint32_t* f
                     sl[q] = e >> 5;
                 }
             }
-            pull_list_scan<NC>(p, L, ls.nb, f_cur, v, sl, serial);
+            // (at 40 registers, the smaller CTAs' limit, a second form would spill)
+            pull_list_scan<NC, T == 1024>(p, L, ls.nb, f_cur, v, sl, serial);
         }
         __syncthreads();
         if (own) {
