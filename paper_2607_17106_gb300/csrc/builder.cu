@@ -362,7 +362,7 @@ __device__ __forceinline__ bool keep_key(uint64_t k, uint64_t prev, bool first, 
 // (on RMAT-22 one lane at a time took 0.5 ms: half the vertices have no larger
 // neighbour).  Warp-uniform.
 __device__ __forceinline__ void fill_rows(int32_t* first, int32_t lo, int32_t hi, int32_t val) {
-    const bool wide = hi - lo >= 4;
+    const bool wide = hi - lo >= 16;
     if (!wide)
         for (int32_t r = lo; r <= hi; ++r) first[r] = val;
     for (unsigned m = __ballot_sync(0xffffffffu, wide); m; m &= m - 1) {
@@ -557,7 +557,8 @@ __global__ void __launch_bounds__(256)
 // cudaMalloc: 2 GB from the stream-ordered pool cost 1.7 ms to map and 3 ms to
 // trim at the next synchronisation, cudaMalloc and cudaFree 0.9 ms.  Up to
 // 32 MB, the least the pool maps, from the pool: builds that follow one
-// another find it still mapped (117 us by cudaMalloc).
+// another find it still mapped (117 us by cudaMalloc), if it is given back
+// after the last wait of a build (a wait trims the pool: 45 us).
 struct Arena {
     cudaStream_t st;
     unsigned char* base = nullptr;
@@ -581,11 +582,13 @@ struct Arena {
         used += pad(std::max<size_t>((size_t)count, 1) * sizeof(T));
         return p;
     }
-    ~Arena() {
-        if (!base) return;
-        if (pooled()) cudaFreeAsync(base, st);
+    void drop() {
+        if (base && pooled()) cudaFreeAsync(base, st);
         else cudaFree(base);
+        base = nullptr;
+        need = used = 0;
     }
+    ~Arena() { drop(); }
 };
 
 enum { ROWS_CSR = 0, ROWS_CSR_CSC = 1, ROWS_SYMMETRIC = 2 };
@@ -620,11 +623,11 @@ struct RowsOut {
 
 // Device arrays of the rows of `count` keys (shape: ROWS_*; ROWS_SYMMETRIC
 // takes KEYS_UNDIRECTED with dedup and drop_self).  With KEYS_ARRAY the key
-// array is used as sort space.  `out` owns nothing after an error.
+// array is used as sort space.  `ar`, empty, takes the scratch: nothing uses
+// it any more when the call returns.  `out` owns nothing after an error.
 bfs_status build_rows(int mode, KeySrc ks, int64_t count, int bits, int dedup, int drop_self, int shape, int32_t n,
-                      cudaStream_t st, RowsOut* out) {
+                      cudaStream_t st, Arena& ar, RowsOut* out) {
     const int64_t tiles = div_up(std::max<int64_t>(count, 1), RS_TILE);
-    Arena ar(st);
     ar.want<uint64_t>(count);
     if (mode != KEYS_ARRAY) ar.want<uint64_t>(count);
     ar.want<uint32_t>(RadixScratch::hist_words(count));
@@ -698,7 +701,7 @@ bfs_status build_rows(int mode, KeySrc ks, int64_t count, int bits, int dedup, i
         }
     }
     if (e == cudaSuccess) e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // the scratch goes now
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
         o.drop();
         return cuda_fail(e, "build rows");
@@ -1025,7 +1028,8 @@ bfs_status rcm_reorder(bfs_graph* g, int bits, cudaStream_t st) {
     relabel_keys_kernel<<<grid_for((int64_t)g->n * 32, 256), 256, 0, st>>>(g->row_ptr, g->col, g->n, g->perm, bits, keys);
     BFS_CUDA(cudaGetLastError());
     RowsOut r;
-    s = build_rows(KEYS_ARRAY, KeySrc{keys, nullptr, nullptr, bits}, g->m, bits, 0, 0, ROWS_CSR, g->n, st, &r);
+    Arena ar(st);
+    s = build_rows(KEYS_ARRAY, KeySrc{keys, nullptr, nullptr, bits}, g->m, bits, 0, 0, ROWS_CSR, g->n, st, ar, &r);
     if (s != BFS_OK) return s;
     take_rows(g, r, true);
     return BFS_OK;
@@ -1083,14 +1087,16 @@ extern "C" bfs_status bfs_build_graph(int32_t n, int64_t m, const int32_t* src, 
     // a kept self-loop of a symmetric graph is two entries, repeats stay
     const bool once = sym && dedup && drop_self;
     RowsOut r;
+    Arena ar(st);
     bfs_status s = build_rows(once ? KEYS_UNDIRECTED : sym ? KEYS_BOTH : KEYS_DIRECTED, ks, once ? m : count, bits, dedup,
-                              drop_self, once ? ROWS_SYMMETRIC : sym ? ROWS_CSR : ROWS_CSR_CSC, n, st, &r);
+                              drop_self, once ? ROWS_SYMMETRIC : sym ? ROWS_CSR : ROWS_CSR_CSC, n, st, ar, &r);
     if (s != BFS_OK) {
         delete g;
         return s;
     }
     take_rows(g, r, sym);
     g->symmetric = sym;
+    if (!ar.pooled() || (flags & (BFS_REORDER_RCM | BFS_PULL_HUBS_FIRST))) ar.drop();
     if (sym && (flags & BFS_REORDER_RCM)) {
         bfs_status sr = rcm_reorder(g, bits, st);
         if (sr != BFS_OK) {
