@@ -440,15 +440,18 @@ __device__ __forceinline__ uint64_t warp_or64(uint64_t x) {
 // lane-major in a warp-uniform loop over the union of the new lanes, so the
 // 32 vertices' entries of one lane's depth row go out together.
 // Dynamic shared memory of the MS-BFS kernel: per warp, the row offset of
-// the parent found for each (lane l, vertex of the warp's word) in a pull
-// level, [l][vertex], so that parents are written lane-major like depths.
-constexpr size_t MS_PIDX_BYTES = (size_t)(MS_T / 32) * 64 * 32 * sizeof(unsigned short);
+// the parent found for each (vertex of the warp's word, lane l) in a pull
+// level, [vertex][l], so that parents are written lane-major like depths.
+// Rows are 66 entries apart: reading one l of 32 vertices, and writing 32 l of
+// one vertex, both hit 32 banks.
+constexpr int MS_PIDX_LD = 66;
+constexpr size_t MS_PIDX_BYTES = (size_t)(MS_T / 32) * 32 * MS_PIDX_LD * sizeof(unsigned short);
 extern __shared__ __align__(16) unsigned short ms_pidx_smem[];
 
 template <bool PAR>
 __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, const uint64_t* f_cur) {
     const unsigned lane = lane_id();
-    unsigned short* pidx = ms_pidx_smem + (threadIdx.x >> 5) * (64 * 32);
+    unsigned short* pidx = ms_pidx_smem + (threadIdx.x >> 5) * (32 * MS_PIDX_LD);
     const int W = (g.n + 31) >> 5;
     const unsigned long long* F = (const unsigned long long*)f_cur;
     // this thread's counters in the push tiles' arrays, not in registers
@@ -518,7 +521,7 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
                     uint64_t b = PAR ? got : 0ull;
                     while (b) {
                         int lj = __ffsll((long long)b) - 1;
-                        pidx[lj * 32 + lane] = (unsigned short)(j - beg);
+                        pidx[lane * MS_PIDX_LD + lj] = (unsigned short)(j - beg);
                         b &= b - 1;
                     }
                 }
@@ -542,37 +545,33 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
                     const int idx = b2 + q * 32 + (int)lane;
                     uu[q] = idx < el ? __ldg(g.csc_col + idx) : -1;
                 }
-                uint64_t mine = 0;
 #pragma unroll
-                for (int q = 0; q < MS_COOP_U; ++q) {
-                    fu[q] = uu[q] >= 0 ? (F[uu[q]] & ml & ~al) : 0ull;
-                    mine |= fu[q];
-                }
-                const uint64_t got = warp_or64(mine);
-                if (PAR && got) {  // warp-uniform
-                    // the first provider of each lane, in entry order: a
-                    // lane's bits that no entry before its own supplies (an
-                    // exclusive OR scan over each group of 32), recorded by
-                    // that lane; a ballot per bit and group took as long
-                    uint64_t before = 0;  // supplied by the groups before
+                for (int q = 0; q < MS_COOP_U; ++q) fu[q] = uu[q] >= 0 ? (F[uu[q]] & ml & ~al) : 0ull;
+                uint64_t got = 0;
+                if (PAR) {
+                    // the entries that supply something new, in entry order;
+                    // thread b records lanes b and b + 32 of each.  A row has
+                    // at most 64 of them and mostly a few: 20 instructions
+                    // each, where an OR scan over the 32 entries of every
+                    // group took 75 and a ballot per lane 16
 #pragma unroll
                     for (int q = 0; q < MS_COOP_U; ++q) {
-                        const uint64_t x = fu[q] & ~before;
-                        if (!__any_sync(0xffffffffu, x != 0)) continue;
-                        uint64_t s = x;
-#pragma unroll
-                        for (int o = 1; o < 32; o <<= 1) {
-                            const uint64_t y = __shfl_up_sync(0xffffffffu, (unsigned long long)s, o);
-                            if ((int)lane >= o) s |= y;
-                        }
-                        const uint64_t ex = __shfl_up_sync(0xffffffffu, (unsigned long long)s, 1);
-                        uint64_t nb = lane ? x & ~ex : x;
-                        before |= __shfl_sync(0xffffffffu, (unsigned long long)s, 31);
-                        while (nb) {
-                            pidx[(__ffsll((long long)nb) - 1) * 32 + l] = (unsigned short)(b2 + q * 32 + (int)lane - bl);
-                            nb &= nb - 1;
+                        uint64_t x = fu[q] & ~got;
+                        for (unsigned m = __ballot_sync(0xffffffffu, x != 0); m; m = __ballot_sync(0xffffffffu, x != 0)) {
+                            const int s = __ffs(m) - 1;
+                            const uint64_t xs = __shfl_sync(0xffffffffu, (unsigned long long)x, s);
+                            const unsigned short at = (unsigned short)(b2 + q * 32 + s - bl);
+                            if (((unsigned)xs >> lane) & 1u) pidx[l * MS_PIDX_LD + lane] = at;
+                            if (((unsigned)(xs >> 32) >> lane) & 1u) pidx[l * MS_PIDX_LD + 32 + lane] = at;
+                            got |= xs;
+                            x &= ~xs;
                         }
                     }
+                } else {
+                    uint64_t mine = 0;
+#pragma unroll
+                    for (int q = 0; q < MS_COOP_U; ++q) mine |= fu[q];
+                    got = warp_or64(mine);
                 }
                 al |= got;
             }
@@ -593,7 +592,7 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
                 all &= all - 1;  // 0 stays 0
                 const bool f = bj[i] >= 0 && ((acc >> bj[i]) & 1ull);
                 if (!f) bj[i] = -1;
-                par[i] = PAR && f ? __ldg(g.csc_col + beg + pidx[bj[i] * 32 + lane]) : 0;
+                par[i] = PAR && f ? __ldg(g.csc_col + beg + pidx[lane * MS_PIDX_LD + bj[i]]) : 0;
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -803,42 +802,50 @@ __device__ __forceinline__ uint64_t* ms_front(const ParamsMS& p, int i) {
 }
 
 // After the last level L of a unit: every depth row written whole.  A warp
-// takes 32 consecutive vertices (lane = vertex) and records, in its
-// shared-memory table [lane j][vertex], the first history level whose mask
-// holds lane j; a lane found only after the history (written as found) is
-// left alone, an unreached one gets -1.  Each lane's 32 entries then go out
-// as one coalesced row segment.  The history masks used are cleared for the
-// next unit.
+// takes 32 consecutive vertices (lane = vertex).  The level of each search
+// lane is gathered in bit planes: plane b holds the lanes found at a history
+// level whose number has bit b, so a level costs a few ORs whatever it found;
+// four lanes' plane bits are then spread over the bytes of a word (a multiply
+// and a mask), all ones for an unreached lane.  A lane found only after the
+// history (written as found) is left alone.  Each lane's 32 entries go out as
+// one coalesced row segment.  The history masks used are cleared for the next
+// unit.  (A byte table in shared memory, filled lane by lane, took twice the
+// instructions.)
 __device__ void ms_depth_pass(const ParamsMS& p, const UnitView& g, MsSmem& sm, int levels) {
     const unsigned lane = lane_id();
-    signed char* tab = (signed char*)(ms_pidx_smem + (threadIdx.x >> 5) * (64 * 32));  // [64][32] int8
     const int lh = min(levels, MS_HIST);
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    const long long ntiles = ((long long)g.n + 31) >> 5;
-    for (long long t = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < ntiles; t += nwarps) {
-        const long long v = t * 32 + lane;
+    const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
+    const int ntiles = (g.n + 31) >> 5;
+    for (int t = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5); t < ntiles; t += nwarps) {
+        const long long v = (long long)t * 32 + lane;
         const bool valid = v < g.n;
-#pragma unroll 4
-        for (int j = 0; j < 64; ++j) tab[j * 32 + lane] = -1;
-        uint64_t found = 0;
-        for (int i = 0; i < lh; ++i) {
-            uint64_t* hp = p.hist + (int64_t)i * p.ncap + v;
-            const uint64_t b = valid ? *hp : 0ull;
-            uint64_t nb = b & ~found;
-            found |= b;
-            while (nb) {
-                const int j = __ffsll((long long)nb) - 1;
-                tab[j * 32 + lane] = (signed char)i;
-                nb &= nb - 1;
+        uint64_t found = 0, pl[4] = {0, 0, 0, 0};
+        for (int i0 = 0; i0 < lh; i0 += 4) {
+            uint64_t b[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) b[i] = valid && i0 + i < lh ? p.hist[(int64_t)(i0 + i) * p.ncap + v] : 0ull;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint64_t nb = b[i] & ~found;
+                found |= b[i];
+                if (i & 1) pl[0] |= nb;
+                if (i & 2) pl[1] |= nb;
+                if (i0 & 4) pl[2] |= nb;
+                if (i0 & 8) pl[3] |= nb;
+                if (b[i]) p.hist[(int64_t)(i0 + i) * p.ncap + v] = 0ull;
             }
-            if (b) *hp = 0ull;
         }
-        const uint64_t later = valid ? (((const unsigned long long*)p.seen)[v] & ~found) : 0ull;
-        __syncwarp();
-        for (int j = 0; j < g.k; ++j) {
-            if (valid && !((later >> j) & 1ull)) sm.depth[j][v] = (int)tab[j * 32 + lane];
+        // lanes found after the history have their depth already
+        const uint64_t skip = levels > MS_HIST && valid ? ((const unsigned long long*)p.seen)[v] & ~found : 0ull;
+        for (int j0 = 0; j0 < g.k; j0 += 4) {
+            const auto spread = [&](uint64_t x) { return (((unsigned)(x >> j0) & 15u) * 0x00204081u) & 0x01010101u; };
+            const unsigned w = spread(pl[0]) | spread(pl[1]) << 1 | spread(pl[2]) << 2 | spread(pl[3]) << 3 |
+                               spread(~found) * 0xffu;
+            const unsigned sk = valid ? (unsigned)(skip >> j0) : 15u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (j0 + i < g.k && !((sk >> i) & 1u)) sm.depth[j0 + i][v] = (int)(signed char)(w >> (8 * i));
         }
-        __syncwarp();
     }
 }
 
