@@ -169,9 +169,19 @@ constexpr int MS_T = 512;
 // memory system fills from DRAM, and every row would first be set to -1.
 constexpr int MS_HIST = 16;
 constexpr int MS_QBUF = 64;       // per-warp staging of active-list appends
-constexpr int MS_LONG_ROW = 1024; // pull rows longer than this are scanned grid-wide
+// Pull rows longer than this are scanned by CTAs after the warps' pass.  A
+// warp stops within a few hundred entries of a hub's row on a dense level, a CTA
+// takes at least 512 and two barriers; but a warp's long scans are the level's
+// tail where every warp has only a word or two.  So the line is low for graphs
+// of at most MS_FEW_WORDS words a warp and high above.  64-lane batches with
+// parents, us, at 512 / 1024 / 2048 / 4096 / 16384: RMAT-16 216 / 246 / 332 / 330 /
+// 444, RMAT-18 456 / 464 / 545 / 555 / 1137, RMAT-19 437 / 380 / 378 / 358 / 356,
+// RMAT-22 2319 / 1958 / 1894 / 1716 / 1679, renumbered without parents 2165 /
+// 1804 / 1740 / 1655 / 1986, RMAT-24 14850 / 11420 / 11440 / 10100 / 9760; 8192: 1725,
+// 1659 and 9820 for the last three.
+constexpr int MS_LONG_ROW_SMALL = 512, MS_LONG_ROW = 8192, MS_FEW_WORDS = 2;
 static_assert(MS_LONG_ROW < 65536, "pull parent positions are staged as 16-bit row offsets");
-constexpr int MS_LONG_ITEMS = 4;  // entries a thread tests per long-row chunk
+constexpr int MS_LONG_ITEMS = 1;  // entries a thread tests per long-row chunk (RMAT-24: 10.08 ms, four 10.14)
 
 #ifndef BFS_MS_PULL_R
 #define BFS_MS_PULL_R 4
@@ -192,6 +202,7 @@ constexpr int MS_PULL_CHUNK = 32, MS_PULL_TAKES = 4;
 struct MsLevelConst {
     int32_t level;
     int pull_chunk;              // pull: words a warp takes at a time
+    int long_row;                // pull: rows longer than this are left to ms_long_rows
     uint64_t* f_next;
     int32_t* a_next;
     int2* u_next;
@@ -484,9 +495,9 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
             beg = __ldg(g.csc_ptr + v);
             end = __ldg(g.csc_ptr + v + 1);
         }
-        // rows longer than MS_LONG_ROW are scanned by the whole grid after
+        // rows longer than long_row are scanned by the whole grid after
         // this pass (ms_long_rows); defer them
-        const bool longrow = miss != 0 && end - beg > MS_LONG_ROW;
+        const bool longrow = miss != 0 && end - beg > L.c.long_row;
         const unsigned lm = __ballot_sync(0xffffffffu, longrow);
         if (lm) {
             unsigned long long base = 0;
@@ -504,29 +515,31 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
         uint64_t acc = 0;
         int j = beg;
         const int lim = min(end, beg + p.pull_serial);
-        // MS_PULL_R entries per step (independent loads), tested in row order
+        // MS_PULL_R entries per step (independent loads), taken in row order;
+        // once every missing lane is found the rest of a step adds nothing
         while (j < lim && acc != miss) {
             int uu[MS_PULL_R];
             uint64_t fm[MS_PULL_R];
 #pragma unroll
             for (int r = 0; r < MS_PULL_R; ++r) uu[r] = j + r < lim ? __ldg(g.csc_col + j + r) : -1;
 #pragma unroll
-            for (int r = 0; r < MS_PULL_R; ++r) fm[r] = uu[r] >= 0 ? F[uu[r]] : 0ull;
+            for (int r = 0; r < MS_PULL_R; ++r) fm[r] = uu[r] >= 0 ? F[uu[r]] & miss : 0ull;
+            if (PAR) {
+                unsigned short* mine = pidx + lane * MS_PIDX_LD;
 #pragma unroll
-            for (int r = 0; r < MS_PULL_R; ++r) {
-                if (uu[r] < 0 || acc == miss) break;
-                const uint64_t got = fm[r] & miss & ~acc;
-                if (got) {
+                for (int r = 0; r < MS_PULL_R; ++r) {
+                    const uint64_t got = fm[r] & ~acc;
                     acc |= got;
-                    uint64_t b = PAR ? got : 0ull;
-                    while (b) {
-                        int lj = __ffsll((long long)b) - 1;
-                        pidx[lane * MS_PIDX_LD + lj] = (unsigned short)(j - beg);
-                        b &= b - 1;
-                    }
+                    // (the halves apart: 32-bit bit scans)
+                    for (unsigned b = (unsigned)got; b; b &= b - 1) mine[__ffs(b) - 1] = (unsigned short)(j + r - beg);
+                    for (unsigned b = (unsigned)(got >> 32); b; b &= b - 1)
+                        mine[__ffs(b) + 31] = (unsigned short)(j + r - beg);
                 }
-                ++j;
+            } else {
+#pragma unroll
+                for (int r = 0; r < MS_PULL_R; ++r) acc |= fm[r];
             }
+            j = min(j + MS_PULL_R, lim);  // the warp goes on from here
         }
         unsigned rm = __ballot_sync(0xffffffffu, miss != 0 && acc != miss && j < end);
         while (rm) {
@@ -579,28 +592,31 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
             rm &= rm - 1;
         }
         // depths and parents of the word, lane-major: for each lane found
-        // anywhere in the word, its row entries of the 32 vertices go out together
-        uint64_t all = PAR || L.c.write_depth ? warp_or64(acc) : 0ull;
+        // anywhere in the word, its row entries of the 32 vertices go out
+        // together.  Four lanes at a time: their parent gathers are in flight
+        // together (one at a time each is a round trip of the word's chain:
+        // RMAT-24 14.17 ms against 13.47), and the lane numbers are constants
+        // but for the group's.
+        const uint64_t all = PAR || L.c.write_depth ? warp_or64(acc) : 0ull;
         __syncwarp();
-        // (four lanes' parent gathers in flight: RMAT-24 14.17 -> 13.47 ms, one at a
-        // time each lane's gather is a round trip of the word's chain)
-        while (all) {  // warp-uniform
-            int bj[4], par[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                bj[i] = all ? __ffsll((long long)all) - 1 : -1;
-                all &= all - 1;  // 0 stays 0
-                const bool f = bj[i] >= 0 && ((acc >> bj[i]) & 1ull);
-                if (!f) bj[i] = -1;
-                par[i] = PAR && f ? __ldg(g.csc_col + beg + pidx[lane * MS_PIDX_LD + bj[i]]) : 0;
+        for (int j0 = 0; all >> j0; j0 += 4) {  // warp-uniform
+            if (!((all >> j0) & 15ull)) {
+                if (j0 == 60) break;
+                continue;
             }
+            const unsigned f = (unsigned)(acc >> j0) & 15u;
+            int par[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                par[i] = PAR && ((f >> i) & 1u) ? __ldg(g.csc_col + beg + pidx[lane * MS_PIDX_LD + j0 + i]) : 0;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                if (bj[i] < 0) continue;
-                if (L.c.write_depth) sm.depth[bj[i]][v] = L.c.level + 1;
-                int32_t* pp = PAR ? sm.parent[bj[i]] : nullptr;
+                if (!((f >> i) & 1u)) continue;
+                if (L.c.write_depth) sm.depth[j0 + i][v] = L.c.level + 1;
+                int32_t* pp = PAR ? sm.parent[j0 + i] : nullptr;
                 if (pp) pp[v] = par[i];
             }
+            if (j0 == 60) break;
         }
         __syncwarp();
         if (acc) {
@@ -1015,8 +1031,10 @@ __device__ void msbfs_body(const ParamsMS& p) {
                 // m_u: degree sum of the vertices some live lane has not seen
                 c.sparse = 8 * m_u < g.m;
                 c.pull_chunk = 1;
+                const int words = (g.n + 31) >> 5, warps = (int)nblocks * (T / 32);
+                c.long_row = words <= MS_FEW_WORDS * warps ? MS_LONG_ROW_SMALL : MS_LONG_ROW;
                 if (c.sparse) {
-                    const int fair = ((g.n + 31) >> 5) / ((int)nblocks * (T / 32) * MS_PULL_TAKES);
+                    const int fair = words / (warps * MS_PULL_TAKES);
                     c.pull_chunk = min(max(fair, 1), MS_PULL_CHUNK);
                 }
             }

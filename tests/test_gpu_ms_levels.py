@@ -57,8 +57,10 @@ def test_batch_levels(kind, k):
     g = bg.Graph.build(n, s, d)
     srcs = np.random.default_rng(k).integers(0, n, k).astype(np.int32)
     ref = [oracle.bfs(adj, int(v), with_parent=False)[0] for v in srcs]
-    # push alone, the heuristic, and alternating forms (pull levels past the history, lists rebuilt); chunk 64: units
-    for o in (dict(policy=bg.BFS_POLICY_PUSH), dict(), dict(schedule=[0, 2, 2, 0, 0], chunk=64)):
+    # push alone, the heuristic, and alternating forms (pull levels past the history, lists rebuilt); chunk 64: units;
+    # pull alone, with serial scans that end inside a step of four
+    for o in (dict(policy=bg.BFS_POLICY_PUSH), dict(), dict(schedule=[0, 2, 2, 0, 0], chunk=64),
+              dict(policy=bg.BFS_POLICY_PULL, pull_serial=3), dict(policy=bg.BFS_POLICY_PULL, pull_serial=1)):
         for par in (True, False):
             depth = torch.full((k, n), -9, dtype=torch.int32, device="cuda")
             parent = torch.full((k, n), -9, dtype=torch.int32, device="cuda") if par else None
