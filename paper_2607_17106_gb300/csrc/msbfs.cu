@@ -211,6 +211,7 @@ struct MsLevelConst {
     unsigned long long* cursor;  // pull: next word to take (zero when the level starts)
     unsigned long long* long_len;  // pull: deferred long rows (zero when the level starts)
     bool sparse;                 // pull: few vertices miss live lanes
+    bool whole;                  // pull: the unit's first; it writes every parent entry not written before
     bool write_depth;            // depths of F_{i+1} are written now (levels past the history)
     bool clear_cur;              // push: F_i's masks are zeroed as they are read (levels past the history)
 };
@@ -483,13 +484,14 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
         // lane (chunk <= 32), where few are open; on a dense level, whose
         // words nearly all have work, the constant bitmap
         const bool mine = (int)lane < min(L.c.pull_chunk, W - w0);
-        const unsigned fl = mine ? (L.c.sparse ? __ldcg(p.full + w0 + lane) : __ldg(g.isolated + w0 + lane)) : 0xffffffffu;
+        const bool whole = PAR && L.c.whole;  // every word
+        const unsigned fl = !mine ? 0xffffffffu : whole ? 0u : L.c.sparse ? __ldcg(p.full + w0 + lane) : __ldg(g.isolated + w0 + lane);
         for (unsigned todo = __ballot_sync(0xffffffffu, fl != 0xffffffffu); todo; todo &= todo - 1) {  // warp-uniform
         const int v = (w0 + __ffs(todo) - 1) * 32 + (int)lane;
         uint64_t miss = 0;
         if (!((__shfl_sync(0xffffffffu, fl, __ffs(todo) - 1) >> lane) & 1u) && v < g.n)
             miss = L.c.live & ~((const unsigned long long*)p.seen)[v];
-        if (!__ballot_sync(0xffffffffu, miss != 0)) continue;
+        if (!whole && !__ballot_sync(0xffffffffu, miss != 0)) continue;
         int beg = 0, end = 0;
         if (miss) {
             beg = __ldg(g.csc_ptr + v);
@@ -597,22 +599,27 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
         // together (one at a time each is a round trip of the word's chain:
         // RMAT-24 14.17 ms against 13.47), and the lane numbers are constants
         // but for the group's.
-        const uint64_t all = PAR || L.c.write_depth ? warp_or64(acc) : 0ull;
+        // The unit's first pull level writes all of a word's entries but those
+        // of lanes that push levels have found: -1 for a lane not found yet.
+        // Rows are then written in whole lines by the level that finds most
+        // entries, and not set to -1 before the search.
+        const uint64_t todo_lanes = whole ? (v < g.n ? ~((const unsigned long long*)p.seen)[v] : 0ull) : acc;
+        const uint64_t all = whole ? g.lanes : PAR || L.c.write_depth ? warp_or64(acc) : 0ull;
         __syncwarp();
         for (int j0 = 0; all >> j0; j0 += 4) {  // warp-uniform
             if (!((all >> j0) & 15ull)) {
                 if (j0 == 60) break;
                 continue;
             }
-            const unsigned f = (unsigned)(acc >> j0) & 15u;
+            const unsigned f = (unsigned)(acc >> j0) & 15u, wr = (unsigned)((todo_lanes & g.lanes) >> j0) & 15u;
             int par[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i)
-                par[i] = PAR && ((f >> i) & 1u) ? __ldg(g.csc_col + beg + pidx[lane * MS_PIDX_LD + j0 + i]) : 0;
+                par[i] = PAR && ((f >> i) & 1u) ? __ldg(g.csc_col + beg + pidx[lane * MS_PIDX_LD + j0 + i]) : -1;
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                if (!((f >> i) & 1u)) continue;
-                if (L.c.write_depth) sm.depth[j0 + i][v] = L.c.level + 1;
+                if (!((wr >> i) & 1u)) continue;
+                if (L.c.write_depth && ((f >> i) & 1u)) sm.depth[j0 + i][v] = L.c.level + 1;
                 int32_t* pp = PAR ? sm.parent[j0 + i] : nullptr;
                 if (pp) pp[v] = par[i];
             }
@@ -824,10 +831,12 @@ __device__ __forceinline__ uint64_t* ms_front(const ParamsMS& p, int i) {
 // four lanes' plane bits are then spread over the bytes of a word (a multiply
 // and a mask), all ones for an unreached lane.  A lane found only after the
 // history (written as found) is left alone.  Each lane's 32 entries go out as
-// one coalesced row segment.  The history masks used are cleared for the next
-// unit.  (A byte table in shared memory, filled lane by lane, took twice the
+// one coalesced row segment.  `parents`: no level has written the parents of
+// the lanes that found nothing.  The history masks used are cleared for the
+// next unit.  (A byte table in shared memory, filled lane by lane, took twice the
 // instructions.)
-__device__ void ms_depth_pass(const ParamsMS& p, const UnitView& g, MsSmem& sm, int levels) {
+template <bool PAR>
+__device__ void ms_depth_pass(const ParamsMS& p, const UnitView& g, MsSmem& sm, int levels, bool parents) {
     const unsigned lane = lane_id();
     const int lh = min(levels, MS_HIST);
     const int nwarps = (int)((gridDim.x * blockDim.x) >> 5);
@@ -861,6 +870,13 @@ __device__ void ms_depth_pass(const ParamsMS& p, const UnitView& g, MsSmem& sm, 
 #pragma unroll
             for (int i = 0; i < 4; ++i)
                 if (j0 + i < g.k && !((sk >> i) & 1u)) sm.depth[j0 + i][v] = (int)(signed char)(w >> (8 * i));
+        }
+        if (PAR && parents) {  // no pull level: -1 where a lane found nothing
+            const uint64_t none = valid ? g.lanes & ~((const unsigned long long*)p.seen)[v] : 0ull;
+            for (uint64_t any = warp_or64(none); any; any &= any - 1) {  // warp-uniform
+                const int j = __ffsll((long long)any) - 1;
+                if (((none >> j) & 1ull) && sm.parent[j]) sm.parent[j][v] = -1;
+            }
         }
     }
 }
@@ -914,12 +930,8 @@ __device__ void msbfs_body(const ParamsMS& p) {
             if (w * 32 + 32 > g.n) bits |= ~((1u << (g.n & 31)) - 1u);
             p.full[w] = bits;
         }
-        // depths are written whole by ms_depth_pass; parents start at -1
-        for (int j = 0; PAR && j < g.k; ++j) {
-            int32_t* pp = sm.parent[j];
-            if (!pp) continue;
-            for (long long v = gtid; v < g.n; v += gthreads) pp[v] = -1;
-        }
+        // depths are written whole by ms_depth_pass, the parents of lanes that
+        // find nothing by the first pull level, or there too
         if (gtid == 0) {
             for (int s = 0; s < 3; ++s) {
                 ctl->slot[s].a_len = 0;
@@ -955,6 +967,7 @@ __device__ void msbfs_body(const ParamsMS& p) {
         int unit_levels = 0;
         int list_valid = 0;  // level whose active list (and chunk units) exists
         bool cnt_ok = false;     // sm.cnt holds the level's counters
+        bool par_set = false;    // every parent entry has been written once
         for (int level = 0;; ++level) {
             CountersMS* cur = &ctl->slot[level % 3];
             CountersMS* nxt = &ctl->slot[(level + 1) % 3];
@@ -1030,6 +1043,7 @@ __device__ void msbfs_body(const ParamsMS& p) {
                 c.long_len = &cur->long_len;
                 // m_u: degree sum of the vertices some live lane has not seen
                 c.sparse = 8 * m_u < g.m;
+                c.whole = PAR && !par_set && dir == BFS_DIR_PULL;
                 c.pull_chunk = 1;
                 const int words = (g.n + 31) >> 5, warps = (int)nblocks * (T / 32);
                 c.long_row = words <= MS_FEW_WORDS * warps ? MS_LONG_ROW_SMALL : MS_LONG_ROW;
@@ -1041,6 +1055,7 @@ __device__ void msbfs_body(const ParamsMS& p) {
             __syncthreads();
             MsLevel L{sm.lv, 0u, 0u, 0u, 0ull, 0};
             const bool pull = dir == BFS_DIR_PULL;
+            par_set |= pull;
             if (pull) ms_pull_level<PAR>(p, g, L, sm, f_cur);
             else ms_push_level<T, PAR>(p, g, L, sm, a_cur, u_cur, f_cur, a, nunits);
             // the level's counters: a share a warp, one atomic each for the CTA
@@ -1105,7 +1120,7 @@ __device__ void msbfs_body(const ParamsMS& p) {
             ++unit_levels;
         }
         // the unit's depth rows; a barrier before the next unit reuses seen
-        ms_depth_pass(p, g, sm, unit_levels);
+        ms_depth_pass<PAR>(p, g, sm, unit_levels, PAR && !par_set);
         if (!grid_sync(&ctl->bar, nblocks, bar_target, p.timeout_ns)) return;
     }
     if (gtid == 0) {
