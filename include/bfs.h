@@ -167,7 +167,11 @@ enum {
  * barrier instead of the grid-wide barrier; the first level that would pull
  * or that has more frontier edges than the cluster's threads, and every level
  * after it, runs in the full persistent kernel (a second launch on the same
- * stream, no host round trip).  Sources run one launch pair each. */
+ * stream, no host round trip).  Sources run one launch pair each.
+ * BFS_SMALL_AUTO also runs whole searches of small graphs of higher degree (up
+ * to about 49,000 vertices with an edge and 2 million entries) in the cluster,
+ * in one launch, unless the launch shape is set or barrier_timeout_ns is below
+ * a millisecond (the hardware barrier takes no limit). */
 enum {
     BFS_SMALL_AUTO = -1, /* on for graphs whose maximum degree is at most 16 (grids, road-like graphs) */
     BFS_SMALL_OFF = 0,

@@ -175,13 +175,13 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
     // A cluster launch keeps the level counters in CTA 0's shared memory
     // (reached by every CTA of the cluster through distributed shared
     // memory) and copies them to the control block when it leaves.
-    __shared__ Counters s_ctr[3];
+    __shared__ Counters s_ctr[CL ? 6 : 1];
     const unsigned warp = threadIdx.x >> 5;
     QueueStage<T>* const qs = reinterpret_cast<QueueStage<T>*>(bfs1_dyn);
     for (int si = 0; si < nsearch; ++si) {
     int32_t* const depth = p.depth + (int64_t)si * p.n;
     int32_t* const parent = p.parent ? p.parent + (int64_t)si * p.n : nullptr;
-    Counters* const cs = CL ? cluster_map_rank0(s_ctr) : ctl->slot + 3 * (si & 1);
+    Counters* const cs = (CL ? cluster_map_rank0(s_ctr) : ctl->slot) + 3 * (si & 1);
     bool s_cnt_ok = false;
     if (p.do_init) {
         const int s = p.srcs ? __ldg(p.srcs + si) : p.src_value;
@@ -296,7 +296,7 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
         // a cluster launch leaves every level but a small push-queue level to
         // the grid-wide launch (the state, m_u as it was before the level, is
         // saved as the loop exits)
-        if (CL && (dir != BFS_DIR_PUSH_QUEUE || e_f > p.small_ef_max || q_valid != level)) {
+        if (CL && !p.small_whole && (dir != BFS_DIR_PUSH_QUEUE || e_f > p.small_ef_max || q_valid != level)) {
             if (level > 0) m_u += e_f;
             break;
         }
@@ -357,11 +357,11 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
         } else if (dir == BFS_DIR_PUSH_QUEUE && q_valid != level) {
             // bitmap -> queue conversion of F_i (after pull levels)
             bitmap_to_queue<T>(p, sm, f_cur, q_cur, u_cur, cur);
-            if (!level_sync<CL>(&ctl->bar, nblocks, bar_target, p.timeout_ns)) return;
-            const unsigned long long* const usrc[1] = {&cur->u_len};
-            unsigned long long uv[1];
-            cta_load_u64<1>(usrc, uv);
-            nunits = (int)uv[0];
+            __shared__ unsigned long long s_units;
+            if (!level_sync<CL>(&ctl->bar, nblocks, bar_target, p.timeout_ns, NoArrivalWork(),
+                                [&]() { s_units = ld_counter<CL>(&cur->u_len); }))
+                return;
+            nunits = (int)s_units;  // written again only behind the level's barrier
             q_valid = level;
         }
         if (gtid == 0) {
@@ -448,9 +448,10 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
     // the next search's init may overwrite P, the queues and the other
     // counter set while slower CTAs are still leaving.
     }  // searches
-    if (CL && gtid == 0) {
+    if constexpr (CL) {
         // the grid-wide launch that continues the search reads them there
-        for (int k = 0; k < 3; ++k) ctl->slot[k] = s_ctr[k];
+        if (gtid == 0 && !p.small_whole)
+            for (int k = 0; k < 3; ++k) ctl->slot[k] = s_ctr[k];
     }
     if (gtid == 0) {
         ctl->next_level = level;
@@ -571,6 +572,33 @@ static int small_levels_for(const bfs_graph* g, const bfs_options& o) {
     if (o.small_levels == BFS_SMALL_OFF) return 0;
     if (o.small_levels == BFS_SMALL_AUTO && g->deg_max > 16) return 0;
     return small_cluster_size();
+}
+
+// Whole searches in the cluster: up to three vertices with an edge for each
+// of its threads.  A level's barrier and counter read take 0.7 us there, 2.0
+// grid-wide, and the launch is cheaper; above, 16 SMs fall behind.  One search,
+// us, grid-wide / cluster: RMAT-10 34.6 / 29.0, RMAT-14 45.4 / 41.4, RMAT-16 (46,000
+// vertices with an edge) 51.1 / 46.8, RMAT-17 57.0 / 60.8; ER of degree 16: 16,384
+// vertices 45.4 / 41.4, 32,768 50.2 / 47.9, 65,536 53.5 / 57.7.
+// The hardware barrier takes no limit: a call that limits its waits to less
+// than such a search may take gets the grid-wide kernel, as does one that asks
+// for a launch shape or no cluster.
+constexpr int64_t SMALL_GRAPH_N = 3 * 16 * SMALL_T, SMALL_GRAPH_M = 1 << 21, SMALL_GRAPH_WAIT_NS = 1000000;
+static int small_graph_for(const bfs_graph* g, const bfs_options& o) {
+    bfs_options d;
+    bfs_options_init(&d);
+    if (o.mode != BFS_MODE_PERSISTENT || o.frontier_sort != BFS_SORT_NONE || o.push_filter != BFS_PUSH_FUSED) return 0;
+    if (o.small_levels != BFS_SMALL_AUTO || o.block_threads != d.block_threads || o.blocks_per_sm != 0) return 0;
+    if (g->n - g->n_isolated > SMALL_GRAPH_N || g->m > SMALL_GRAPH_M || g->n > 4 * SMALL_GRAPH_N) return 0;
+    if (o.barrier_timeout_ns < SMALL_GRAPH_WAIT_NS || g->deg_max <= 16) return 0;
+    return small_cluster_size();
+}
+
+static cudaError_t run_small_graph(Params1 q, int cl, cudaStream_t st) {
+    q.do_init = 1;
+    q.level_count = INT32_MAX / 2;
+    q.small_whole = 1;
+    return launch_small(q, cl, st);
 }
 
 // The small levels by bfs_small.cu: maximum degree at most 8, and a direction
@@ -830,7 +858,9 @@ bfs_status run_single(bfs_graph* g, int32_t src_value, int32_t* depth, int32_t* 
     } else {
         p.do_init = 1;
         p.level_count = INT32_MAX / 2;
-        if (const int cl = small_levels_for(g, o)) {
+        if (const int cl = small_graph_for(g, o)) {
+            BFS_CUDA(run_small_graph(p, cl, st));
+        } else if (const int cl = small_levels_for(g, o)) {
             // the small levels in one cluster, the rest grid-wide (a launch
             // that finds the search done returns at once)
             BFS_CUDA(run_small_pair(g, w, o, p, cl, launcher, st));
@@ -886,6 +916,11 @@ bfs_status run_single_many(bfs_graph* g, const int32_t* src_host, int32_t k, int
     CoopLauncher launcher(o);
     if (o.frontier_sort == BFS_SORT_DEVICE && launcher.blocks > 4096)
         return fail(BFS_EINVAL, "frontier_sort supports at most 4096 CTAs (launch has %d)", launcher.blocks);
+    if (const int cl = small_graph_for(g, o)) {
+        BFS_CUDA(cudaMemsetAsync(w->ctl, 0, sizeof(Ctl1), st));
+        BFS_CUDA(run_small_graph(p, cl, st));
+        return BFS_OK;
+    }
     if (const int cl = small_levels_for(g, o)) {
         // a pair of launches per source: the small levels in one cluster,
         // the rest grid-wide

@@ -6,7 +6,8 @@ hand a queue to the push level after them, hubs with chunk units among it;
 frontiers with less and with more than half of the edges (two forms of the pull
 scan); unreached and isolated entries in dirty output rows off a 16-byte
 boundary.  Depths and the level count against the oracle, parents validated,
-several searches in one launch and one at a time.
+several searches in one launch and one at a time, in the cluster (automatic
+for graphs of this size) and grid-wide.
 """
 import ctypes
 
@@ -48,7 +49,7 @@ def _case(kind):
 
 
 @pytest.mark.parametrize("kind", ["rmat16", "er-connected", "er-sparse", "complete", "late-hub", "ba"])
-@pytest.mark.parametrize("opt", [dict(), dict(chunk=64), dict(block_threads=512), dict(mode=bg.BFS_MODE_HOST_LOOP),
+@pytest.mark.parametrize("opt", [dict(), dict(small_levels=bg.BFS_SMALL_OFF), dict(small_levels=bg.BFS_SMALL_OFF, chunk=64), dict(chunk=64), dict(block_threads=512), dict(mode=bg.BFS_MODE_HOST_LOOP),
                                  dict(alpha=0.001, beta=1e9), dict(alpha=1e9, beta=1e-6)])
 def test_last_levels(kind, opt):
     from paper_2607_17106_gb300 import build
