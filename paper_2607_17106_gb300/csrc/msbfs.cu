@@ -1263,7 +1263,16 @@ static bfs_status launch_ms(WorkspaceMS* w, const std::vector<MsUnit>& units, co
     for (const MsUnit& u : units)
         for (int j = 0; j < u.k; ++j) par |= u.parent[j] != nullptr;
     const void* kernel = par ? (const void*)msbfs_kernel<MS_T, true> : (const void*)msbfs_kernel<MS_T, false>;
-    int blocks = coop_blocks_ms(kernel, o.blocks_per_sm);
+    // Little work a level: one CTA an SM, for the shorter barrier.  Entries
+    // bound a dense level's work; on bounded-degree graphs a level is a
+    // frontier's worth, vertices times lanes over a long diameter.  us, two
+    // CTAs / one: RMAT-12 79 / 68, RMAT-15 247 / 234, RMAT-16 262 / 272, RMAT-17 230 /
+    // 275; grids with 4 lanes, 400^2 6054 / 5429, 1000^2 14393 / 12824, with 48,
+    // 700^2 12549 / 12645, 1000^2 22289 / 22959.
+    bool light = true;
+    for (const MsUnit& u : units)
+        light &= u.m <= (1 << 20) || (u.deg_max <= 16 && (int64_t)u.n * u.k <= (1 << 24));
+    int blocks = coop_blocks_ms(kernel, light && o.blocks_per_sm == 0 ? 1 : o.blocks_per_sm);
     void* args[] = {(void*)&p};
     BFS_CUDA(cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(MS_T), args, MS_PIDX_BYTES,
                                          st));
