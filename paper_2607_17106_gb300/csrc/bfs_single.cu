@@ -679,7 +679,7 @@ static bfs_status ensure_ws1(bfs_graph* g, int32_t chunk, cudaStream_t st, Works
              cudaMalloc(&w->U[i], w->ucap * sizeof(int2)) == cudaSuccess;
     }
     ok = ok && cudaMalloc(&w->ctl, sizeof(Ctl1)) == cudaSuccess;
-    ok = ok && cudaMalloc(&w->d_sticky, 4) == cudaSuccess && cudaMemset(w->d_sticky, 0, 4) == cudaSuccess;
+    ok = ok && cudaMalloc(&w->d_sticky, 4) == cudaSuccess && cudaMemsetAsync(w->d_sticky, 0, 4, st) == cudaSuccess;
     ok = ok && cudaMallocHost(&w->h_ctl, sizeof(Ctl1)) == cudaSuccess;
     if (!ok) {
         free_ws1(w);

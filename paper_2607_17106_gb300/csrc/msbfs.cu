@@ -1167,7 +1167,11 @@ static int64_t count_units(bfs_graph* g, int32_t chunk, cudaStream_t st) {
     return (int64_t)h;
 }
 
-static bfs_status alloc_wsms(int32_t ncap, int64_t ucap, int32_t chunk, int32_t units_cap, WorkspaceMS** out) {
+// The zeroing is ordered on the stream of the launch that uses the workspace
+// first (on the default stream it would not be ordered before a launch on a
+// non-blocking one).
+static bfs_status alloc_wsms(int32_t ncap, int64_t ucap, int32_t chunk, int32_t units_cap, cudaStream_t st,
+                             WorkspaceMS** out) {
     WorkspaceMS* w = new (std::nothrow) WorkspaceMS();
     if (!w) return fail(BFS_ENOMEM, "host allocation");
     w->ncap = ncap;
@@ -1180,14 +1184,14 @@ static bfs_status alloc_wsms(int32_t ncap, int64_t ucap, int32_t chunk, int32_t 
              cudaMalloc(&w->act[i], (size_t)ncap * 4) == cudaSuccess &&
              cudaMalloc(&w->U[i], (size_t)ucap * sizeof(int2)) == cudaSuccess;
     ok = ok && cudaMalloc(&w->ctl, sizeof(CtlMS)) == cudaSuccess;
-    ok = ok && cudaMalloc(&w->d_sticky, 4) == cudaSuccess && cudaMemset(w->d_sticky, 0, 4) == cudaSuccess;
+    ok = ok && cudaMalloc(&w->d_sticky, 4) == cudaSuccess && cudaMemsetAsync(w->d_sticky, 0, 4, st) == cudaSuccess;
     ok = ok && cudaMalloc(&w->d_units, sizeof(MsUnit) * (size_t)units_cap) == cudaSuccess;
     ok = ok && cudaMalloc(&w->longv, (size_t)ncap * 4) == cudaSuccess;
     ok = ok && cudaMalloc(&w->acc_long, (size_t)ncap * 8) == cudaSuccess;
     ok = ok && cudaMalloc(&w->hist, (size_t)MS_HIST * ncap * 8) == cudaSuccess &&
-         cudaMemset(w->hist, 0, (size_t)MS_HIST * ncap * 8) == cudaSuccess;
+         cudaMemsetAsync(w->hist, 0, (size_t)MS_HIST * ncap * 8, st) == cudaSuccess;
     ok = ok && cudaMalloc(&w->full, (size_t)div_up(ncap, 32) * 4) == cudaSuccess;
-    ok = ok && cudaMalloc(&w->hist_dirty, 4) == cudaSuccess && cudaMemset(w->hist_dirty, 0, 4) == cudaSuccess;
+    ok = ok && cudaMalloc(&w->hist_dirty, 4) == cudaSuccess && cudaMemsetAsync(w->hist_dirty, 0, 4, st) == cudaSuccess;
     ok = ok && cudaMallocHost(&w->h_ctl, sizeof(CtlMS)) == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -1292,7 +1296,7 @@ bfs_status run_msbfs(bfs_graph* g, const int32_t* sources, int32_t k, int32_t* d
         }
         int64_t uc = count_units(g, o.chunk, st);
         if (uc < 0) return fail(BFS_ECUDA, "unit count");
-        bfs_status s = alloc_wsms(g->n, uc + 64, o.chunk, std::max(nunits, 4), &w);
+        bfs_status s = alloc_wsms(g->n, uc + 64, o.chunk, std::max(nunits, 4), st, &w);
         if (s != BFS_OK) return s;
         g->wsms = w;
     }
@@ -1400,7 +1404,7 @@ bfs_status run_mixed(const bfs_graph* const* graphs, int32_t n_graphs, const int
         w = big->wsmix = nullptr;
     }
     if (!w) {
-        s = alloc_wsms(big->n, ucap, o.chunk, (int32_t)units.size(), &w);
+        s = alloc_wsms(big->n, ucap, o.chunk, (int32_t)units.size(), st, &w);
         if (s != BFS_OK) return s;
         if (kept.owns_lock()) big->wsmix = w;
     }

@@ -372,7 +372,8 @@ extern "C" bfs_status bfs_policy_load(const float* weights, int32_t nw, bfs_poli
               cudaMalloc(&p->m2, NPARAM * 4) == cudaSuccess && cudaMalloc(&p->grad, NPARAM * 4) == cudaSuccess &&
               cudaMalloc(&p->loss, 4) == cudaSuccess;
     if (ok) ok = cudaMemcpy(p->w, p->host.data(), NWEIGHTS * 4, cudaMemcpyHostToDevice) == cudaSuccess &&
-                 cudaMemset(p->m1, 0, NPARAM * 4) == cudaSuccess && cudaMemset(p->m2, 0, NPARAM * 4) == cudaSuccess;
+                 cudaMemset(p->m1, 0, NPARAM * 4) == cudaSuccess && cudaMemset(p->m2, 0, NPARAM * 4) == cudaSuccess &&
+                 cudaStreamSynchronize(nullptr) == cudaSuccess;  // zero for a step on any stream
     if (!ok) {
         cudaGetLastError();
         bfs_policy_free(p);
