@@ -25,8 +25,8 @@
 // common.cuh.  What bounds it is the gathers: per vertex a row-offset pair, two
 // column sectors and a few label hops, which stay in L2 (67 MB for 2^24
 // vertices); 64 warps an SM (32 registers a thread) hide them.  Measured
-// around the call: RMAT-22 3,283 -> 286 us, the 4096^2 grid 135-180 ms
-// (2,800 to 3,400 iterations) -> 2.7 ms.
+// around the call: RMAT-22 3,283 -> 134 us, the 4096^2 grid 135-180 ms
+// (2,800 to 3,400 iterations) -> 1.2 ms, ER-22 2.2 -> 0.35 ms.
 #include "common.cuh"
 
 #include <algorithm>
@@ -42,6 +42,8 @@ constexpr int CC_HOPS = 32;      // parents a vertex climbs in one shortcut pass
 constexpr int CC_SAMPLES = 1024; // labels looked at to find the largest tree
 constexpr int CC_SLOTS = 2048;   // hash slots they are counted in
 constexpr int CC_WARP_ROW = 16;  // longer rows are hooked by a whole warp
+constexpr int CC_HUB = 256;      // a hub's row reaches 1 / CC_HUB of the vertices
+constexpr int CC_LOOKS = 2;      // looks at the last neighbours before they are hooked, without hubs
 constexpr int CC_BIG_ROW = 4096; // rows of at least this many entries by the whole grid
 
 struct CtlCC {
@@ -60,18 +62,25 @@ struct ParamsCC {
     CtlCC* ctl;
     int32_t* big;       // their vertices, m / CC_BIG_ROW + 1
     int32_t big_cap;
+    int32_t many_trees; // no hubs: first neighbours leave many trees
     int64_t timeout_ns;
 };
 
+// Labels are read through L1 (ld.ca): the roots of large trees are read by
+// every warp, and in L2 those reads queue on a few sectors (the 4096^2 grid's
+// hooks of last neighbours took 2.3 ms, RMAT-22 in all 250 us instead of 110).
+// A stale label is an older parent of the same vertex, and a hook is decided
+// by its CAS; barriers make the labels of earlier phases visible.
+//
 // Root of v's tree.  Every vertex on the way is pointed past its parent: a
 // plain store is safe, because only a root is ever hooked (by CAS) and a
 // vertex that has a parent keeps one; whichever of two racing stores lands
 // last, it names an ancestor.  Ends: each hop goes to a smaller id.
 __device__ __forceinline__ int cc_find(int32_t* L, int v) {
     int prev = v;
-    int p = __ldcg(L + v);
+    int p = __ldca(L + v);
     while (p != prev) {
-        const int g = __ldcg(L + p);
+        const int g = __ldca(L + p);
         if (g == p) break;
         __stcg(L + prev, g);
         prev = p;
@@ -107,12 +116,12 @@ __device__ bool cc_shortcut(const ParamsCC& p, unsigned& bar_target, int& pass, 
         unsigned* open = &p.ctl->open[pass % 3];
         bool left = false;
         for (long long v = gtid; v < p.n; v += gthreads) {
-            const int own = __ldcg(p.label + v);
+            const int own = __ldca(p.label + v);
             int r = own, g = own;
             bool root = false;
 #pragma unroll 1
             for (int k = 0; k < CC_HOPS; ++k) {
-                g = __ldcg(p.label + r);
+                g = __ldca(p.label + r);
                 if (g == r) {
                     root = true;
                     break;
@@ -160,14 +169,34 @@ __global__ void __launch_bounds__(CC_T, 4) cc_kernel(ParamsCC p) {
     ++iters;
     if (!grid_sync(&ctl->bar, gridDim.x, bar_target, p.timeout_ns)) return;
     if (!cc_shortcut(p, bar_target, pass, iters)) return;
-    // the last neighbour of every row (a row's only entry is done if smaller)
-    for (long long v = gtid; v < p.n; v += gthreads) {
-        const int b = __ldg(p.row_ptr + v), e = __ldg(p.row_ptr + v + 1);
-        if (b == e) continue;
-        const int u = __ldg(p.col + e - 1);
-        if (e - b >= 2 || u > (int)v) cc_hook(L, cc_find(L, (int)v), u);
+    // The last neighbour of every row (a row's only entry is done if smaller).
+    // Without hubs there are still many trees, and a million hooks at once keep
+    // losing their CAS to one another.  A look at the edge then only lowers the
+    // larger root's label to the smallest root seen beside it (one atomicMin, no
+    // search; the labels are roots, and only roots' are written).  What such a
+    // root was joined to before may be lost again, but every edge is hooked
+    // properly afterwards, when most have one root.
+    for (int look = p.many_trees ? CC_LOOKS : 0; look >= 0; --look) {
+        for (long long v = gtid; v < p.n; v += gthreads) {
+            const int b = __ldg(p.row_ptr + v), e = __ldg(p.row_ptr + v + 1);
+            if (b == e) continue;
+            const int u = __ldg(p.col + e - 1);
+            if (e - b < 2 && u < (int)v) continue;
+            const int x = __ldca(L + v), y = __ldca(L + u);
+            if (x == y) continue;
+            if (look > 0) {
+                const int hi = max(x, y), lo = min(x, y);
+                if (lo < __ldca(L + hi)) atomicMin(L + hi, lo);
+            } else {
+                cc_hook(L, cc_find(L, x), y);
+            }
+        }
+        ++iters;
+        if (look > 0) {
+            if (!grid_sync(&ctl->bar, gridDim.x, bar_target, p.timeout_ns)) return;
+            if (!cc_shortcut(p, bar_target, pass, iters)) return;
+        }
     }
-    ++iters;
     if (!grid_sync(&ctl->bar, gridDim.x, bar_target, p.timeout_ns)) return;
     if (!cc_shortcut(p, bar_target, pass, iters)) return;
 
@@ -181,7 +210,7 @@ __global__ void __launch_bounds__(CC_T, 4) cc_kernel(ParamsCC p) {
     __syncthreads();
     for (int i = threadIdx.x; i < CC_SAMPLES; i += CC_T) {
         const unsigned long long h = (unsigned long long)(unsigned)i * 2654435761ull + 12345ull;
-        const int l = __ldcg(L + (long long)(h % (unsigned long long)p.n));
+        const int l = __ldca(L + (long long)(h % (unsigned long long)p.n));
         unsigned s = ((unsigned)l * 2654435761u) >> 21;  // 11 bits: CC_SLOTS
         for (int tries = 0; tries < CC_SLOTS; ++tries, s = (s + 1) & (CC_SLOTS - 1)) {
             const int old = atomicCAS(&s_key[s], -1, l);
@@ -210,7 +239,7 @@ __global__ void __launch_bounds__(CC_T, 4) cc_kernel(ParamsCC p) {
     for (long long v0 = gtid - lane; v0 < p.n; v0 += gthreads) {  // warp-uniform
         const long long v = v0 + lane;
         int b = 0, e = 0;
-        if (v < p.n && __ldcg(L + v) != giant) {
+        if (v < p.n && __ldca(L + v) != giant) {
             b = __ldg(p.row_ptr + v);
             e = __ldg(p.row_ptr + v + 1) - 1;
         }
@@ -223,7 +252,7 @@ __global__ void __launch_bounds__(CC_T, 4) cc_kernel(ParamsCC p) {
             int a = cc_find(L, (int)v);
             for (int j = b; j < e; ++j) {
                 const int u = __ldg(p.col + j);
-                if (__ldcg(L + u) != a) a = cc_hook(L, a, u);
+                if (__ldca(L + u) != a) a = cc_hook(L, a, u);
             }
         }
         unsigned wm = __ballot_sync(0xffffffffu, len > CC_WARP_ROW && len < CC_BIG_ROW - 1);
@@ -234,7 +263,7 @@ __global__ void __launch_bounds__(CC_T, 4) cc_kernel(ParamsCC p) {
             int a = cc_find(L, (int)(v0 + l));
             for (int j = bl + (int)lane; j < el; j += 32) {
                 const int u = __ldg(p.col + j);
-                if (__ldcg(L + u) != a) a = cc_hook(L, a, u);
+                if (__ldca(L + u) != a) a = cc_hook(L, a, u);
             }
             __syncwarp();
         }
@@ -243,13 +272,13 @@ __global__ void __launch_bounds__(CC_T, 4) cc_kernel(ParamsCC p) {
     if (!grid_sync(&ctl->bar, gridDim.x, bar_target, p.timeout_ns)) return;
     const int nb = min(*(volatile int*)&ctl->n_big, p.big_cap);
     for (int i = 0; i < nb; ++i) {
-        const int v = __ldcg(p.big + i);
+        const int v = __ldca(p.big + i);
         const int b = __ldg(p.row_ptr + v), e = __ldg(p.row_ptr + v + 1) - 1;
         if (b + gtid < e) {
             int a = cc_find(L, v);
             for (long long j = b + gtid; j < e; j += gthreads) {
                 const int u = __ldg(p.col + j);
-                if (__ldcg(L + u) != a) a = cc_hook(L, a, u);
+                if (__ldca(L + u) != a) a = cc_hook(L, a, u);
             }
         }
     }
@@ -300,6 +329,12 @@ extern "C" bfs_status bfs_components(const bfs_graph* gc, int32_t* label, int32_
     p.ctl = (CtlCC*)g->cc_scratch;
     p.big = (int32_t*)(p.ctl + 1);
     p.big_cap = big_cap;
+    // A matter of time alone; us around the call with 0 / 1 / 2 / 3 looks:
+    // RMAT-22 134 / 171 / 211 / 252 (a hub), with a = 0.45 and edge factor 8 300 /
+    // 199 / 246 / 283 (none); ER-22 607 / 803 / 348 / 407, 2^17 vertices of degree
+    // 8 195 / 328 / 76 / 83; grids 4096^2 1085 / 1083 / 1156 / 1217, 1000^2 583 /
+    // 318 / 233 / 424.
+    p.many_trees = (int64_t)g->deg_max * CC_HUB < n;
     p.timeout_ns = 2000000000ll;
     int per_sm = 0;
     CtlCC h{};
