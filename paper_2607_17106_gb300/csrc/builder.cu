@@ -286,10 +286,13 @@ int radix_chunk(int64_t tiles) { return (int)std::max<int64_t>(1, std::min<int64
 struct RadixScratch {
     uint32_t *hist = nullptr, *chunk = nullptr, *total = nullptr;
     static int64_t hist_words(int64_t count) { return div_up(std::max<int64_t>(count, 1), RS_TILE) * RS_BINS; }
+    // The chunks of any sort of at most `count` keys, not of `count` alone: with
+    // c < RS_CHUNK tiles a chunk there are fewer than (c + 1) * radix_ctas()
+    // tiles, so at most 2 * radix_ctas() chunks (1215 tiles take 1215 at 608
+    // CTAs, 1216 take 608).
     static int64_t chunk_words(int64_t count) {
         const int64_t tiles = div_up(std::max<int64_t>(count, 1), RS_TILE);
-        // of every sort of fewer keys too: see radix_chunk
-        return std::max(div_up(tiles, radix_chunk(tiles)), std::min(tiles, radix_ctas() + 1)) * RS_BINS;
+        return std::max(div_up(tiles, RS_CHUNK), std::min(tiles, 2 * radix_ctas())) * RS_BINS;
     }
     template <typename S>
     cudaError_t alloc(S& sc, int64_t count) {

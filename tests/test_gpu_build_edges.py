@@ -95,3 +95,15 @@ def test_ids_out_of_range(bad, flags):
         with pytest.raises(bg.BfsError) as err:
             bg.Graph.build(5, e[0], e[1], flags=flags)
         assert err.value.status == bg.BFS_EINVAL
+
+
+# Counting CTAs take 1, 2, .. 8 tiles, by the tiles of the sort over the CTAs
+# there are: the second sort, of the keys kept, can have more chunks than the first.
+@pytest.mark.parametrize("first,kept", [(2.0, 1.99), (2.0, 1.5), (3.01, 1.99), (3.01, 0.5)])
+@pytest.mark.parametrize("flags", [SYM | DEDUP | DROP | CSC, DEDUP | DROP | CSC])
+def test_second_sort_of_fewer_keys(first, kept, flags):
+    ctas = 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    m, k = int(first * ctas * 6144) + 1, int(kept * ctas * 6144)
+    s, d = _edges("uniform", 1 << 18, k, 11)
+    r = np.arange(m) % k  # the rest repeats edges
+    _check(1 << 18, s[r], d[r], flags, device=True)
