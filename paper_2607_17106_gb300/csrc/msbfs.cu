@@ -663,8 +663,7 @@ __device__ void ms_long_rows(const ParamsMS& p, const UnitView& g, MsSmem& sm, c
         const uint64_t miss = live & ~((const unsigned long long*)p.seen)[v];
         if (threadIdx.x == 0) s_or = 0;
         __syncthreads();
-        for (int lo = beg; lo < end; lo += per) {
-            if ((s_or & miss) == miss) break;  // CTA-uniform: read after the barrier below
+        for (int lo = beg; lo < end && miss; lo += per) {  // CTA-uniform
             const int hi = min(end, lo + per);
 #pragma unroll
             for (int k = 0; k < MS_LONG_ITEMS; ++k) {
@@ -684,6 +683,11 @@ __device__ void ms_long_rows(const ParamsMS& p, const UnitView& g, MsSmem& sm, c
                 }
             }
             __syncthreads();
+            // every thread looks before any adds to s_or again: a thread that
+            // saw the next step's lanes would leave a step before the others
+            const bool all = s_or == miss;
+            __syncthreads();
+            if (all) break;
         }
         const uint64_t acc = s_or;
         if (threadIdx.x == 0) p.acc_long[r] = acc;

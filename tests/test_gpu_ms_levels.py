@@ -71,3 +71,36 @@ def test_batch_levels(kind, k):
                 assert np.array_equal(got[j], ref[j]), (o, j)
                 if par and j % 9 == 0:
                     assert oracle.validate(adj, int(srcs[j]), ref[j], parent[j].cpu().numpy()) == 0
+
+
+# Rows above MS_LONG_ROW_SMALL entries, scanned by a CTA in steps of 512: hubs
+# joined to the same `width` vertices, their missing lanes complete in the
+# first, the last or no step.
+@pytest.mark.parametrize("width", [511, 512, 513, 1024, 4099, 9001])
+@pytest.mark.parametrize("k", [1, 64, 96])
+def test_long_rows(width, k):
+    from paper_2607_17106_gb300 import build
+    build.build()
+    hubs = 300
+    n = hubs + width + 40
+    rng = np.random.default_rng(width + k)
+    s = np.repeat(np.arange(hubs, dtype=np.int32), width)
+    d = (hubs + np.tile(np.arange(width), hubs)).astype(np.int32)
+    tail = np.arange(hubs + width, n, dtype=np.int32)  # a path into one end of the rows
+    s, d = np.concatenate([s, tail[:-1], tail[-1:]]), np.concatenate([d, tail[1:], np.int32([n - 41])])
+    adj = oracle.build_adjacency(n, s, d)
+    g = bg.Graph.build(n, s, d)
+    srcs = rng.integers(0, n, k).astype(np.int32)
+    ref = {v: oracle.bfs(adj, v, with_parent=False)[0] for v in set(srcs.tolist())}
+    for o in (dict(policy=bg.BFS_POLICY_PULL), dict()):
+        for par in (True, False):
+            depth = torch.full((k, n), -9, dtype=torch.int32, device="cuda")
+            parent = torch.full((k, n), -9, dtype=torch.int32, device="cuda") if par else None
+            g.run(srcs, depth, parent, bg.options(batch=1, **o))
+            g.sync()
+            got = depth.cpu().numpy()
+            for j, v in enumerate(srcs.tolist()):
+                assert np.array_equal(got[j], ref[v]), (o, j)
+                if par and j % 9 == 0:
+                    assert oracle.validate(adj, v, ref[v], parent[j].cpu().numpy()) == 0
+    g.free()
