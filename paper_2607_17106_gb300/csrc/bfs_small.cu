@@ -22,7 +22,7 @@
 //   - depth and parent of a vertex are stored when its entry is expanded, at
 //     the start of the next level, and are done long before its barrier.
 // A level takes 2.0 us up to 2 M cells (OR and row 0.7 us, cluster barrier 0.7,
-// append 0.3, counters 0.3) and 3.4 us on the 4096^2 grid, whose rows and outputs
+// append 0.3, counters 0.3) and 2.8 us on the 4096^2 grid, whose rows and outputs
 // (400 MB touched at random by one cluster) miss L2 and the TLB: a search
 // of that grid 41.7 -> 19.2 ms.
 // The level that would not fit, or that is not a push-queue level, is handed
