@@ -6,7 +6,7 @@
 // general kernel the chain is: queue entry (L2), column (HBM), visited OR (L2)
 // with the new vertex's row bounds (HBM), queue reservation, store drain,
 // barrier -- 6.2 us a level on the relabelled 4096^2 grid.  Here it is one
-// memory round trip and the cluster's hardware barrier:
+// memory round trip and one message between the CTAs:
 //   - adjacency in rows of W = 4 or 8 entries (-1 for none), one aligned
 //     sector a vertex, built once per graph.  A candidate's row is loaded
 //     beside the OR that claims it, and the claimer puts it in the queue
@@ -18,13 +18,18 @@
 //     receiver, and every CTA expands the same share of the next frontier
 //     wherever the wavefront runs (a CTA that kept its own claims would keep
 //     its patch of it).  The claim counts are pushed to every CTA the same
-//     way, so that after the barrier all reads are local;
+//     way, so that all of a level's reads are local;
+//   - the stores signal the level themselves: they are asynchronous and
+//     counted by an mbarrier of the receiver (two, in turn: a sender is at most
+//     a level ahead), and each sender arrives there with the bytes it has
+//     stored.  A cluster barrier waits for every store before it, those to
+//     memory too, and took 0.35 us a level more;
 //   - depth and parent of a vertex are stored when its entry is expanded, at
-//     the start of the next level, and are done long before its barrier.
-// A level takes 2.0 us up to 2 M cells (OR and row 0.7 us, cluster barrier 0.7,
-// append 0.3, counters 0.3) and 2.8 us on the 4096^2 grid, whose rows and outputs
-// (400 MB touched at random by one cluster) miss L2 and the TLB: a search
-// of that grid 41.7 -> 19.2 ms.
+//     the start of the next level, and nothing waits for them.
+// A level takes 1.7 us up to 2 M cells (OR and row 0.7 us, append 0.3, the
+// message and the CTA barriers the rest) and 3.1 us on the 4096^2 grid, whose rows
+// and outputs (400 MB touched at random by one cluster) miss L2 and the TLB: a
+// search of that grid 41.7 -> 18.2 ms.
 // The level that would not fit, or that is not a push-queue level, is handed
 // to the grid-wide kernel with the state that kernel continues from.
 #include "level.cuh"
@@ -36,6 +41,7 @@ namespace bfsgb {
 namespace {
 
 constexpr int ELL_T = 1024;
+constexpr long long ELL_WAIT_NS = 1000000000ll;  // a level's wait is never given up earlier
 
 template <int W>
 struct EllCfg {
@@ -66,11 +72,47 @@ __device__ __forceinline__ unsigned map_shared(const void* p, unsigned rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void st_cluster2(unsigned a, int x, int y) {
-    asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
+// Stores to a CTA's shared memory that its mbarrier `bar` counts, in bytes, as they land
+__device__ __forceinline__ void st_async2(unsigned a, int x, int y, unsigned bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b32 [%0], {%1, %2}, [%3];" ::"r"(a), "r"(x),
+                 "r"(y), "r"(bar)
+                 : "memory");
 }
-__device__ __forceinline__ void st_cluster(unsigned a, unsigned x) {
-    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(a), "r"(x) : "memory");
+__device__ __forceinline__ void st_async(unsigned a, unsigned x, unsigned bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(a), "r"(x), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void mbar_init(unsigned long long* b, int arrivals) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(b)), "r"(arrivals)
+                 : "memory");
+}
+// One arrival at a CTA's mbarrier, with the bytes this CTA's stores bring it.
+// Relaxed: a release waits for the CTA's depth and parent stores, which no one
+// reads here (2.17 us a level against 1.67).  What the receiver reads are the
+// counted stores alone; the sender's own reads of the queue part that is
+// written next were used, and its ORs on P returned, before this.
+__device__ __forceinline__ void mbar_arrive_tx(unsigned bar, unsigned bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes)
+                 : "memory");
+}
+__device__ __forceinline__ bool mbar_try(unsigned bar, unsigned parity) {
+    unsigned ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// false: the limit has passed
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, int64_t limit_ns) {
+    if (mbar_try(bar, parity)) return true;
+    const uint64_t t0 = globaltimer_ns();
+    while (!mbar_try(bar, parity))
+        if ((int64_t)(globaltimer_ns() - t0) > limit_ns) return false;
+    return true;
 }
 __device__ __forceinline__ void cluster_sync() {
     __syncwarp();
@@ -103,12 +145,14 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
     extern __shared__ __align__(16) int32_t ell_q[];  // [2][cl][PART][PITCH]
     __shared__ unsigned s_cnt[2][16];                 // packed claims of each CTA, by level parity
     __shared__ unsigned s_mine[2];                    // this CTA's, being counted
+    __shared__ unsigned long long s_bar[2];           // a level's arrivals and bytes, by level parity
     const int cl = (int)gridDim.x, lg = __ffs(cl) - 1, rank = (int)cluster_rank();
     const int lane = (int)lane_id();
     const int grp = (int)threadIdx.x / W, j = (int)threadIdx.x % W;
     const int per = C::GROUPS / cl;            // groups that expand the entries of one sender
     const int from = grp / per, r = grp % per; // warp-uniform sender: per * W >= 32
     Ctl1* ctl = p.ctl;
+    const int64_t limit_ns = max((long long)p.timeout_ns, ELL_WAIT_NS);
 
     if (threadIdx.x < 32) {
         const int s = p.src_value;
@@ -119,6 +163,9 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
         __syncwarp();
         if (lane == 0) {
             s_mine[0] = s_mine[1] = 0;
+            mbar_init(&s_bar[0], cl);
+            mbar_init(&s_bar[1], cl);
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
             int row[W], deg = 0;
             ell_row(p.ell, s, row);
 #pragma unroll
@@ -184,6 +231,7 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
                                  (rank - from) & (cl - 1), lg);
         const int32_t* q = ell_q + ((size_t)par * cl + from) * C::PART * C::PITCH;
         int32_t* qn = ell_q + ((size_t)(par ^ 1) * cl + rank) * C::PART * C::PITCH;  // this CTA's part, at any receiver
+        unsigned long long* const bar = &s_bar[par ^ 1];
         for (int i0 = 0; i0 < len; i0 += per) {  // warp-uniform
             int u = -1, w = -1;
             if (i0 + r < len) {
@@ -218,19 +266,36 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
             base = __shfl_sync(0xffffffffu, base, 0) & ((1u << CNT_BITS) - 1u);
             if (won) {
                 const int k = (int)base + __popc(cm & lanemask_lt());
-                const unsigned a = map_shared(qn + (k >> lg) * C::PITCH, (unsigned)((rank + k) & (cl - 1)));
-                st_cluster2(a, w, u);
+                const unsigned to = (unsigned)((rank + k) & (cl - 1));
+                const unsigned a = map_shared(qn + (k >> lg) * C::PITCH, to), b = map_shared(bar, to);
+                st_async2(a, w, u, b);
 #pragma unroll
-                for (int t = 0; t < W; t += 2) st_cluster2(a + 8 + 4 * t, row[t], row[t + 1]);
+                for (int t = 0; t < W; t += 2) st_async2(a + 8 + 4 * t, row[t], row[t + 1], b);
             }
         }
         __syncthreads();  // every claim of the CTA is counted
-        if (threadIdx.x < (unsigned)cl)
-            st_cluster(map_shared(&s_cnt[par ^ 1][rank], threadIdx.x), s_mine[par]);
+        if (threadIdx.x < (unsigned)cl) {
+            const unsigned to = threadIdx.x, m = s_mine[par], b = map_shared(bar, to);
+            const int sent = part_len((int)(m & ((1u << CNT_BITS) - 1u)), ((int)to - rank) & (cl - 1), lg);
+            st_async(map_shared(&s_cnt[par ^ 1][rank], to), m, b);
+            mbar_arrive_tx(b, (unsigned)(sent * C::PITCH * (int)sizeof(int32_t)) + 4u);
+        }
         if (threadIdx.x == 32) s_mine[par ^ 1] = 0;  // pushed a level ago, counts the next one
         f_prev = f;
-        cluster_sync();
+        bool ok = true;
+        if (threadIdx.x < 32) {
+            ok = mbar_wait((unsigned)__cvta_generic_to_shared(bar), (level >> 1) & 1, limit_ns);
+            __syncwarp();
+        }
+        if (!__syncthreads_and(ok)) {  // CTA-uniform; the other CTAs' waits end the same way
+            if (threadIdx.x == 0) atomicCAS(&ctl->bar.err, 0, (int)DEV_TIMEOUT);
+            f = 0;
+            done = true;
+            break;
+        }
     }
+    // No CTA leaves before all have stopped sending.
+    cluster_sync();
     // The frontier F_level that was not expanded: depths and parents, and the
     // queue entries of the grid-wide kernel.  Nothing is left of a finished one.
     if (f > 0) {
