@@ -290,9 +290,12 @@ __device__ __forceinline__ void ms_emit(const ParamsMS& p, MsLevel& L, MsSmem& s
 
 // Push candidate u -> v with frontier lanes fu: the lanes of fu that v has not
 // seen are ORed into seen[v], whose old value names exactly one claimer per
-// (v, lane); the claimer enters them in F_{i+1}[v] and writes their parent
-// (and depth).  Returns true for the first entry into F_{i+1}[v], with v's
-// degree in deg.
+// (v, lane), which writes the lane's parent (and depth), and into F_{i+1}[v].
+// The read of seen[v] is no older than the level (the barrier before it), so a
+// lane in it that another thread claims first is claimed in this level and
+// belongs in F_{i+1}[v] all the same: both ORs, and the row bounds of v, are in
+// flight together.  Returns true for the first entry into F_{i+1}[v] (some
+// lane of it may be another thread's), with v's degree in deg.
 template <bool PAR>
 __device__ __forceinline__ bool ms_claim(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, bool has, int v,
                                          int u, uint64_t fu, int& deg) {
@@ -302,15 +305,16 @@ __device__ __forceinline__ bool ms_claim(const ParamsMS& p, const UnitView& g, M
     if (has) bits = fu & ~((const unsigned long long*)p.seen)[v];
     if (!bits) return false;
     const uint64_t old = atomicOr((unsigned long long*)p.seen + v, (unsigned long long)bits);
+    const uint64_t in = atomicOr((unsigned long long*)L.c.f_next + v, (unsigned long long)bits);
+    const int rb = __ldg(g.row_ptr + v), re = __ldg(g.row_ptr + v + 1);
     const uint64_t nb = bits & ~old, now = old | bits;
-    if (!nb) return false;
-    const uint64_t in = atomicOr((unsigned long long*)L.c.f_next + v, (unsigned long long)nb);
-    L.lanes |= nb;
-    if (PAR || L.c.write_depth) write_lanes(sm, nb, v, u, L.c.level + 1, L.c.write_depth);
-    const bool done = (now & L.c.live) == L.c.live && (old & L.c.live) != L.c.live;
-    if (in == 0 || done) deg = __ldg(g.row_ptr + v + 1) - __ldg(g.row_ptr + v);
-    if (done) L.done_e += (unsigned)deg;
-    if (now == g.lanes) atomicOr(p.full + (v >> 5), 1u << (v & 31));
+    deg = re - rb;
+    if (nb) {
+        L.lanes |= nb;
+        if (PAR || L.c.write_depth) write_lanes(sm, nb, v, u, L.c.level + 1, L.c.write_depth);
+        if ((now & L.c.live) == L.c.live && (old & L.c.live) != L.c.live) L.done_e += (unsigned)deg;
+        if (now == g.lanes) atomicOr(p.full + (v >> 5), 1u << (v & 31));
+    }
     return in == 0;
 }
 
