@@ -70,7 +70,7 @@ struct WorkspaceMS {
     int32_t chunk = 0;
     uint64_t* seen = nullptr;
     uint64_t* front[2] = {nullptr, nullptr};
-    int32_t* act[2] = {nullptr, nullptr};
+    int4* act[2] = {nullptr, nullptr};
     int2* U[2] = {nullptr, nullptr};
     CtlMS* ctl = nullptr;
     int* d_sticky = nullptr;
@@ -121,8 +121,8 @@ struct ParamsMS {
     uint64_t* seen;
     uint64_t* F0;
     uint64_t* F1;
-    int32_t* A0;
-    int32_t* A1;
+    int4* A0;  // active lists: vertex, row begin, row end, 0
+    int4* A1;
     int2* U0;
     int2* U1;
     int64_t ucap;
@@ -157,6 +157,7 @@ struct UnitView {
     int32_t n;
     int32_t k;
     int32_t symmetric;
+    int32_t deg_max;
     uint64_t lanes;
 };
 
@@ -168,7 +169,7 @@ constexpr int MS_T = 512;
 // entries are scattered 4-byte stores into partly written sectors, which the
 // memory system fills from DRAM, and every row would first be set to -1.
 constexpr int MS_HIST = 16;
-constexpr int MS_QBUF = 64;       // per-warp staging of active-list appends
+constexpr int MS_QBUF = 128;      // per-warp staging of active-list appends
 // Pull rows longer than this are scanned by CTAs after the warps' pass.  A
 // warp stops within a few hundred entries of a hub's row on a dense level, a CTA
 // takes at least 512 and two barriers; but a warp's long scans are the level's
@@ -204,7 +205,7 @@ struct MsLevelConst {
     int pull_chunk;              // pull: words a warp takes at a time
     int long_row;                // pull: rows longer than this are left to ms_long_rows
     uint64_t* f_next;
-    int32_t* a_next;
+    int4* a_next;
     int2* u_next;
     CountersMS* next;
     uint64_t live;               // lanes with a non-empty frontier F_i
@@ -227,7 +228,6 @@ struct MsSmem {
     int src[MS_T];
     unsigned long long fmask[MS_T];
     int scan_tmp[33];
-    int32_t qbuf[(MS_T / 32) * MS_QBUF];
     float feat[BFS_MLP_IN];
     float mlp_out;
     unsigned long long red[4][MS_T / 32];  // a level's e_f, |F|, done_e and lanes, one share a warp
@@ -247,6 +247,23 @@ struct MsLevel {
     int qn;                  // staged appends (warp-uniform)
 };
 
+// Dynamic shared memory of the MS-BFS kernel: per warp, the row offset of
+// the parent found for each (vertex of the warp's word, lane l) in a pull
+// level, [vertex][l], so that parents are written lane-major like depths.
+// Rows are 66 entries apart: reading one l of 32 vertices, and writing 32 l of
+// one vertex, both hit 32 banks.
+constexpr int MS_PIDX_LD = 66;
+constexpr size_t MS_PIDX_BYTES = (size_t)(MS_T / 32) * 32 * MS_PIDX_LD * sizeof(unsigned short);
+extern __shared__ __align__(16) unsigned short ms_pidx_smem[];
+// A push level stages a warp's active-list appends in the same bytes (MS_QBUF
+// vertices, row begins and row ends), all there is without parents.  What
+// the CTAs do not take is L1, which dense pulls gather masks through: with the
+// staging in bytes of its own (196 KB of shared memory an SM, not 164) RMAT-24
+// took 8.86 ms with parents against 8.10.
+constexpr size_t MS_QBUF_BYTES = (size_t)(MS_T / 32) * 3 * MS_QBUF * sizeof(int32_t);
+static_assert(MS_QBUF_BYTES <= MS_PIDX_BYTES, "staging fits the parent offsets' bytes");
+__device__ __forceinline__ int32_t* ms_qbuf() { return (int32_t*)ms_pidx_smem + (threadIdx.x >> 5) * 3 * MS_QBUF; }
+
 __device__ __forceinline__ void write_lanes(MsSmem& sm, uint64_t bits, int v, int par, int d, bool write_depth) {
     while (bits) {
         int j = __ffsll((long long)bits) - 1;
@@ -261,27 +278,32 @@ __device__ __forceinline__ void ms_units(const ParamsMS& p, int2* u_out, Counter
 }
 
 __device__ __forceinline__ void ms_flush(MsLevel& L, MsSmem& sm) {
-    const int32_t* qbuf = sm.qbuf + (threadIdx.x >> 5) * MS_QBUF;
+    const int32_t* qbuf = ms_qbuf();
     if (L.qn == 0) return;
     unsigned lane = lane_id();
     unsigned long long base = 0;
     if (lane == 0) base = atomicAdd(&L.c.next->a_len, (unsigned long long)L.qn);
     base = __shfl_sync(0xffffffffu, base, 0);
     __syncwarp();
-    for (int i = (int)lane; i < L.qn; i += 32) L.c.a_next[base + i] = qbuf[i];
+    for (int i = (int)lane; i < L.qn; i += 32) L.c.a_next[base + i] = make_int4(qbuf[i], qbuf[MS_QBUF + i], qbuf[2 * MS_QBUF + i], 0);
     __syncwarp();
     L.qn = 0;
 }
 
-// v entered F_{i+1} (first OR into its mask this level): stage it for the
-// active list, add its degree, split big rows into chunk units.  Warp-uniform.
-__device__ __forceinline__ void ms_emit(const ParamsMS& p, MsLevel& L, MsSmem& sm, bool first, int v, int deg) {
+// v entered F_{i+1} (first OR into its mask this level): stage it and its row
+// bounds for the active list, add its degree, split big rows into chunk units.  Warp-uniform.
+__device__ __forceinline__ void ms_emit(const ParamsMS& p, MsLevel& L, MsSmem& sm, bool first, int v, int rb,
+                                        int re) {
     unsigned cm = __ballot_sync(0xffffffffu, first);
     if (!cm) return;
     int c = __popc(cm);
     if (L.qn + c > MS_QBUF) ms_flush(L, sm);
     if (first) {
-        sm.qbuf[(threadIdx.x >> 5) * MS_QBUF + L.qn + __popc(cm & lanemask_lt())] = v;
+        const int deg = re - rb;
+        int32_t* slot = ms_qbuf() + L.qn + __popc(cm & lanemask_lt());
+        slot[0] = v;
+        slot[MS_QBUF] = rb;
+        slot[2 * MS_QBUF] = re;
         L.ef += (unsigned)deg;
         if (deg >= p.chunk) ms_units(p, L.c.u_next, L.c.next, v, deg);
     }
@@ -295,10 +317,10 @@ __device__ __forceinline__ void ms_emit(const ParamsMS& p, MsLevel& L, MsSmem& s
 // lane in it that another thread claims first is claimed in this level and
 // belongs in F_{i+1}[v] all the same: both ORs, and the row bounds of v, are in
 // flight together.  Returns true for the first entry into F_{i+1}[v] (some
-// lane of it may be another thread's), with v's degree in deg.
+// lane of it may be another thread's), with v's row bounds in rb, re.
 template <bool PAR>
 __device__ __forceinline__ bool ms_claim(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, bool has, int v,
-                                         int u, uint64_t fu, int& deg) {
+                                         int u, uint64_t fu, int& rb, int& re) {
     uint64_t bits = 0;
     // an ordinary load: hubs are read by thousands of threads, which the L1 then
     // serves; lanes only grow, so a stale word costs an OR at most
@@ -306,13 +328,13 @@ __device__ __forceinline__ bool ms_claim(const ParamsMS& p, const UnitView& g, M
     if (!bits) return false;
     const uint64_t old = atomicOr((unsigned long long*)p.seen + v, (unsigned long long)bits);
     const uint64_t in = atomicOr((unsigned long long*)L.c.f_next + v, (unsigned long long)bits);
-    const int rb = __ldg(g.row_ptr + v), re = __ldg(g.row_ptr + v + 1);
+    rb = __ldg(g.row_ptr + v);
+    re = __ldg(g.row_ptr + v + 1);
     const uint64_t nb = bits & ~old, now = old | bits;
-    deg = re - rb;
     if (nb) {
         L.lanes |= nb;
         if (PAR || L.c.write_depth) write_lanes(sm, nb, v, u, L.c.level + 1, L.c.write_depth);
-        if ((now & L.c.live) == L.c.live && (old & L.c.live) != L.c.live) L.done_e += (unsigned)deg;
+        if ((now & L.c.live) == L.c.live && (old & L.c.live) != L.c.live) L.done_e += (unsigned)(re - rb);
         if (now == g.lanes) atomicOr(p.full + (v >> 5), 1u << (v & 31));
     }
     return in == 0;
@@ -321,9 +343,9 @@ __device__ __forceinline__ bool ms_claim(const ParamsMS& p, const UnitView& g, M
 template <bool PAR>
 __device__ __forceinline__ void ms_candidate(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, bool has,
                                              int v, int u, uint64_t fu) {
-    int deg = 0;
-    const bool first = ms_claim<PAR>(p, g, L, sm, has, v, u, fu, deg);
-    ms_emit(p, L, sm, first, v, deg);
+    int rb = 0, re = 0;
+    const bool first = ms_claim<PAR>(p, g, L, sm, has, v, u, fu, rb, re);
+    ms_emit(p, L, sm, first, v, rb, re);
 }
 
 // End of a push level: the warps' staged appends, with one atomic for the CTA
@@ -342,53 +364,55 @@ __device__ void ms_flush_all(MsLevel& L, MsSmem& sm) {
     if (total == 0) return;
     if (threadIdx.x == 0) sm.base = atomicAdd(&L.c.next->a_len, (unsigned long long)total);
     __syncthreads();
-    for (int i = lane; i < L.qn; i += 32) L.c.a_next[sm.base + before + i] = sm.qbuf[warp * MS_QBUF + i];
+    const int32_t* qbuf = ms_qbuf();
+    for (int i = lane; i < L.qn; i += 32)
+        L.c.a_next[sm.base + before + i] = make_int4(qbuf[i], qbuf[MS_QBUF + i], qbuf[2 * MS_QBUF + i], 0);
     L.qn = 0;
 }
 
+// A tile of the active list, one entry a thread (vertex < 0: none).  An entry
+// carries its row's bounds, and a candidate loads its source's mask beside its
+// column, so between the entry and the first ORs there are two round trips
+// (the 2048 x 1531 grid with 32 lanes 44.4 -> 41.6 ms).
 template <int T, bool PAR>
-__device__ void ms_push_tile(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, int u, uint64_t* f_cur) {
+__device__ void ms_push_tile(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, int4 e, uint64_t* f_cur) {
     static_assert(T <= MS_T, "tile arrays are sized for MS_T threads");
     unsigned lane = lane_id();
-    int beg = 0, end = 0;
-    uint64_t fu = 0;
-    if (u >= 0) {
-        beg = __ldg(g.row_ptr + u);
-        end = __ldg(g.row_ptr + u + 1);
-        fu = f_cur[u];
-        if (end - beg >= p.chunk) end = beg;  // chunk units cover it
-        else if (L.c.clear_cur) f_cur[u] = 0;   // read once, by this thread
-    }
+    const unsigned long long* F = (const unsigned long long*)f_cur;
+    const int u = e.x, beg = e.y;
+    int end = e.z;
+    const bool unit = end - beg >= p.chunk;
+    if (unit) end = beg;  // chunk units cover it
     // medium rows: 32-edge segments taken in turn by every warp of the CTA
-    const bool med = (end - beg) >= p.medium;
-    int nseg_total;
-    const int soff = block_exclusive_scan(med ? (end - beg + 31) >> 5 : 0, sm.scan_tmp, &nseg_total);
-    if (nseg_total > 0) {
-        sm.off[threadIdx.x] = soff;
-        sm.beg[threadIdx.x] = beg;
-        sm.lim[threadIdx.x] = end;
-        sm.src[threadIdx.x] = u;
-        sm.fmask[threadIdx.x] = fu;
-        __syncthreads();
-        for (int s = (int)(threadIdx.x >> 5); s < nseg_total; s += T / 32) {
-            int lo = 0, hi = T - 1;
-            while (lo < hi) {
-                int mid = (lo + hi + 1) >> 1;
-                if (sm.off[mid] <= s) lo = mid; else hi = mid - 1;
+    if (g.deg_max >= p.medium) {
+        const bool med = (end - beg) >= p.medium;
+        int nseg_total;
+        const int soff = block_exclusive_scan(med ? (end - beg + 31) >> 5 : 0, sm.scan_tmp, &nseg_total);
+        if (nseg_total > 0) {
+            sm.off[threadIdx.x] = soff;
+            sm.beg[threadIdx.x] = beg;
+            sm.lim[threadIdx.x] = end;
+            sm.src[threadIdx.x] = u;
+            __syncthreads();
+            for (int s = (int)(threadIdx.x >> 5); s < nseg_total; s += T / 32) {
+                int lo = 0, hi = T - 1;
+                while (lo < hi) {
+                    int mid = (lo + hi + 1) >> 1;
+                    if (sm.off[mid] <= s) lo = mid; else hi = mid - 1;
+                }
+                const int j = sm.beg[lo] + ((s - sm.off[lo]) << 5) + (int)lane;
+                const bool has = j < sm.lim[lo];
+                const int v = has ? __ldg(g.col + j) : 0;
+                ms_candidate<PAR>(p, g, L, sm, has, v, sm.src[lo], F[sm.src[lo]]);
             }
-            const int j = sm.beg[lo] + ((s - sm.off[lo]) << 5) + (int)lane;
-            const bool has = j < sm.lim[lo];
-            const int v = has ? __ldg(g.col + j) : 0;
-            ms_candidate<PAR>(p, g, L, sm, has, v, sm.src[lo], sm.fmask[lo]);
         }
+        if (med) end = beg;
     }
-    if (med) end = beg;
-    int deg = end - beg, total;
-    int off = block_exclusive_scan(deg, sm.scan_tmp, &total);
+    int total;
+    int off = block_exclusive_scan(end - beg, sm.scan_tmp, &total);
     sm.off[threadIdx.x] = off;
     sm.beg[threadIdx.x] = beg;
     sm.src[threadIdx.x] = u;
-    sm.fmask[threadIdx.x] = fu;
     if (threadIdx.x == T - 1) sm.off[T] = total;
     __syncthreads();
     for (int k0 = 0; k0 < total; k0 += T) {
@@ -403,18 +427,20 @@ __device__ void ms_push_tile(const ParamsMS& p, const UnitView& g, MsLevel& L, M
                 if (sm.off[mid] <= k) lo = mid; else hi = mid - 1;
             }
             su = sm.src[lo];
-            sf = sm.fmask[lo];
             v = __ldg(g.col + sm.beg[lo] + (k - sm.off[lo]));
+            sf = F[su];
         }
         ms_candidate<PAR>(p, g, L, sm, has, v, su, sf);
     }
     __syncthreads();
+    // the mask has been read, by this tile alone
+    if (L.c.clear_cur && u >= 0 && !unit) f_cur[u] = 0;
 }
 
 // Push level: items = chunk units of big rows, then CTA tiles of the active
 // list, dealt round-robin over the CTAs.
 template <int T, bool PAR>
-__device__ void ms_push_level(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, const int32_t* a_cur,
+__device__ void ms_push_level(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, const int4* a_cur,
                               const int2* u_cur, uint64_t* f_cur, long long a, long long nunits) {
     long long per_tile = (a + gridDim.x - 1) / gridDim.x;
     per_tile = per_tile < 1 ? 1 : (per_tile > T ? T : per_tile);
@@ -434,8 +460,8 @@ __device__ void ms_push_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
             }
         } else {
             long long q = (it - nunits) * per_tile + threadIdx.x;
-            int u = (threadIdx.x < per_tile && q < a) ? a_cur[q] : -1;
-            ms_push_tile<T, PAR>(p, g, L, sm, u, f_cur);
+            const int4 e = (threadIdx.x < per_tile && q < a) ? a_cur[q] : make_int4(-1, 0, 0, 0);
+            ms_push_tile<T, PAR>(p, g, L, sm, e, f_cur);
         }
     }
     ms_flush_all<T>(L, sm);
@@ -455,14 +481,6 @@ __device__ __forceinline__ uint64_t warp_or64(uint64_t x) {
 // `pull_serial` entries are finished by the whole warp.  Depths are written
 // lane-major in a warp-uniform loop over the union of the new lanes, so the
 // 32 vertices' entries of one lane's depth row go out together.
-// Dynamic shared memory of the MS-BFS kernel: per warp, the row offset of
-// the parent found for each (vertex of the warp's word, lane l) in a pull
-// level, [vertex][l], so that parents are written lane-major like depths.
-// Rows are 66 entries apart: reading one l of 32 vertices, and writing 32 l of
-// one vertex, both hit 32 banks.
-constexpr int MS_PIDX_LD = 66;
-constexpr size_t MS_PIDX_BYTES = (size_t)(MS_T / 32) * 32 * MS_PIDX_LD * sizeof(unsigned short);
-extern __shared__ __align__(16) unsigned short ms_pidx_smem[];
 
 template <bool PAR>
 __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, const uint64_t* f_cur) {
@@ -747,7 +765,7 @@ __device__ void ms_long_finalize(const ParamsMS& p, const UnitView& g, MsSmem& s
 // here (after a pull level the next push has at most a few per cent of the
 // vertices), so reading the masks is the cost.  (A block scan per 512 masks took
 // 100 us for the 2^24 vertices of RMAT-24.)
-__device__ void ms_masks_to_list(const ParamsMS& p, const UnitView& g, const uint64_t* f_cur, int32_t* a_cur,
+__device__ void ms_masks_to_list(const ParamsMS& p, const UnitView& g, const uint64_t* f_cur, int4* a_cur,
                                  int2* u_cur, CountersMS* cur) {
     constexpr int R = 8;
     const unsigned lane = lane_id();
@@ -775,9 +793,9 @@ __device__ void ms_masks_to_list(const ParamsMS& p, const UnitView& g, const uin
         for (int r = 0; r < R; ++r) {
             if (m[r]) {
                 const int v = (int)(v0 + r * 32 + lane);
-                a_cur[at + __popc(b[r] & lanemask_lt())] = v;
-                const int deg = __ldg(g.row_ptr + v + 1) - __ldg(g.row_ptr + v);
-                if (deg >= p.chunk) ms_units(p, u_cur, cur, v, deg);
+                const int rb = __ldg(g.row_ptr + v), re = __ldg(g.row_ptr + v + 1);
+                a_cur[at + __popc(b[r] & lanemask_lt())] = make_int4(v, rb, re, 0);
+                if (re - rb >= p.chunk) ms_units(p, u_cur, cur, v, re - rb);
             }
             at += __popc(b[r]);
         }
@@ -919,6 +937,7 @@ __device__ void msbfs_body(const ParamsMS& p) {
             g.n = U->n;
             g.k = U->k;
             g.symmetric = U->symmetric;
+            g.deg_max = U->deg_max;
             g.lanes = (U->k >= 64) ? ~0ull : ((1ull << U->k) - 1);
         }
         int deg_max = U->deg_max;
@@ -962,9 +981,9 @@ __device__ void msbfs_body(const ParamsMS& p) {
             unsigned long long old = atomicOr((unsigned long long*)ms_front(p, 0) + s, 1ull << j);
             if (sm.parent[j]) sm.parent[j][s] = s;
             if (old == 0) {
-                int deg = g.row_ptr[s + 1] - g.row_ptr[s];
+                const int rb = g.row_ptr[s], re = g.row_ptr[s + 1], deg = re - rb;
                 unsigned long long idx = atomicAdd(&ctl->slot[0].a_len, 1ull);
-                p.A0[idx] = s;
+                p.A0[idx] = make_int4(s, rb, re, 0);
                 atomicAdd(&ctl->slot[0].e_f, (unsigned long long)deg);
                 if (deg >= p.chunk) ms_units(p, p.U0, &ctl->slot[0], s, deg);
             }
@@ -1012,7 +1031,7 @@ __device__ void msbfs_body(const ParamsMS& p) {
                 r.t_ns = (int64_t)globaltimer_ns();
                 p.log[level] = r;
             }
-            int32_t* a_cur = (level & 1) ? p.A1 : p.A0;
+            int4* a_cur = (level & 1) ? p.A1 : p.A0;
             int2* u_cur = (level & 1) ? p.U1 : p.U0;
             uint64_t* f_cur = ms_front(p, level);
             long long nunits = (long long)cv[3];
@@ -1189,7 +1208,7 @@ static bfs_status alloc_wsms(int32_t ncap, int64_t ucap, int32_t chunk, int32_t 
     bool ok = cudaMalloc(&w->seen, (size_t)ncap * 8) == cudaSuccess;
     for (int i = 0; i < 2 && ok; ++i)
         ok = cudaMalloc(&w->front[i], (size_t)ncap * 8) == cudaSuccess &&
-             cudaMalloc(&w->act[i], (size_t)ncap * 4) == cudaSuccess &&
+             cudaMalloc(&w->act[i], (size_t)ncap * sizeof(int4)) == cudaSuccess &&
              cudaMalloc(&w->U[i], (size_t)ucap * sizeof(int2)) == cudaSuccess;
     ok = ok && cudaMalloc(&w->ctl, sizeof(CtlMS)) == cudaSuccess;
     ok = ok && cudaMalloc(&w->d_sticky, 4) == cudaSuccess && cudaMemsetAsync(w->d_sticky, 0, 4, st) == cudaSuccess;
@@ -1210,10 +1229,10 @@ static bfs_status alloc_wsms(int32_t ncap, int64_t ucap, int32_t chunk, int32_t 
     return BFS_OK;
 }
 
-static int coop_blocks_ms(const void* kernel, int blocks_per_sm) {
+static int coop_blocks_ms(const void* kernel, size_t smem, int blocks_per_sm) {
     int per_sm = 0;
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MS_PIDX_BYTES);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, MS_T, MS_PIDX_BYTES);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, MS_T, smem);
     if (per_sm < 1) per_sm = 1;
     if (blocks_per_sm > 0) per_sm = std::min(per_sm, blocks_per_sm);
     return per_sm * num_sms();
@@ -1284,10 +1303,10 @@ static bfs_status launch_ms(WorkspaceMS* w, const std::vector<MsUnit>& units, co
     bool light = true;
     for (const MsUnit& u : units)
         light &= u.m <= (1 << 20) || (u.deg_max <= 16 && (int64_t)u.n * u.k <= (1 << 24));
-    int blocks = coop_blocks_ms(kernel, light && o.blocks_per_sm == 0 ? 1 : o.blocks_per_sm);
+    const size_t smem = par ? MS_PIDX_BYTES : MS_QBUF_BYTES;
+    int blocks = coop_blocks_ms(kernel, smem, light && o.blocks_per_sm == 0 ? 1 : o.blocks_per_sm);
     void* args[] = {(void*)&p};
-    BFS_CUDA(cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(MS_T), args, MS_PIDX_BYTES,
-                                         st));
+    BFS_CUDA(cudaLaunchCooperativeKernel(kernel, dim3(blocks), dim3(MS_T), args, smem, st));
     return BFS_OK;
 }
 
