@@ -780,7 +780,7 @@ def main():
                                               extra_flags=bg.BFS_PULL_HUBS_FIRST)
 
     if not args.no_extra:
-        # connected components by min-label propagation on the same graph
+        # connected components of the same graph
         lab = torch.empty(n, dtype=torch.int32, device="cuda")
         g.components(lab)
         times, iters = [], 0

@@ -270,7 +270,7 @@ bfs_status bfs_sync(const bfs_graph* g, void* cuda_stream);
  * entries; depth/parent are host arrays of nq device pointers (parent or its
  * entries may be NULL).  Queries are grouped per graph into 64-lane units and
  * the units are handed out to CTA teams by a device work counter.
- * The workspace (about 190 bytes a vertex of the largest graph in the batch)
+ * The workspace (about 200 bytes a vertex of the largest graph in the batch)
  * stays with that graph and is freed with it; a call that finds it in use by
  * another thread's call makes its own.
  * Errors as bfs_run.

@@ -133,7 +133,7 @@ __device__ __forceinline__ bool level_sync(GridBarrier* b, unsigned nblocks, uns
 // A pull level that can find only few vertices (their degrees sum to at most
 // m_u) appends them to the next queue as it finds them: the push level that
 // follows (f < n / beta) then needs no pass over the bitmap and no barrier for
-// it (RMAT-22's sixth level 10.3 -> XX us).
+// it (64 searches of RMAT-22 8.00 -> 7.89 ms).
 __device__ __forceinline__ bool pull_appends(const Params1& p, long long m_u) {
     return p.symmetric && p.policy == BFS_POLICY_HEURISTIC && 256 * m_u <= (long long)p.n;
 }

@@ -415,9 +415,9 @@ bool ell_prepare(const bfs_graph* g, Workspace1* w, cudaStream_t st) {
 }
 
 // Rows are loaded with the candidates while they fit in L2 (126 MB): on a
-// 1000^2 grid 2.24 us a level against 2.32, on the 4096^2 grid (268 MB of rows, two
-// thirds of the loads for vertices visited before) 3.85 against 3.57, equal
-// at 2900^2 (134 MB).
+// 1000^2 grid 1.69 us a level against 1.74, on the 4096^2 grid (268 MB of rows, two
+// thirds of the loads for vertices visited before) 3.46 against 3.10, near
+// equal at 2900^2 (134 MB: 2.21, 2.28).
 static bool ell_speculate(const bfs_graph* g, int width) {
     return (int64_t)g->n * width * (int64_t)sizeof(int32_t) <= ((int64_t)128 << 20);
 }

@@ -186,9 +186,9 @@ __device__ inline int decide_dir(const Params1& p, int level, long long f, long 
 // rows make a few frontier words very hot, which the L1 then serves.
 
 // ------------------------------------------------------------ claiming
-// Per-warp shared-memory staging of next-queue entries (64: every flush is an
-// atomic on the one queue counter; ER-22's widest push level has a million
-// appends, 15.26 -> 14.83 ms for 64 searches).
+// Per-warp shared-memory staging of next-queue entries.  Every flush is an
+// atomic on the one queue counter, and ER-22's widest push level has a million
+// appends: 64 searches 15.26 ms with 64 entries, 14.83 with 128.
 constexpr int QBUF = 128;
 
 struct LevelCtx {
