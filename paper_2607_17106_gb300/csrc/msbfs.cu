@@ -183,6 +183,14 @@ constexpr int MS_QBUF = 128;
 // 1659 and 9820 for the last three.
 constexpr int MS_LONG_ROW_SMALL = 512, MS_LONG_ROW = 8192, MS_FEW_WORDS = 2;
 static_assert(MS_LONG_ROW < 65536, "pull parent positions are staged as 16-bit row offsets");
+// Row entries a warp scans together in the 32 rows of a word before it leaves
+// what is left of them to CTAs.  Lanes that none of a word of hubs can find yet
+// (renumbered graphs have such words) would otherwise keep one warp for
+// milliseconds: RMAT-19 renumbered, 5 lanes, one seed 1258 us without a limit,
+// 412 / 443 / 499 at 16384 / 24576 / 32768; RMAT-22 renumbered x 64 2227 us against
+// 1641 / 1674 / 1714; RMAT-24 x 64 8.08 ms against 8.28 / 8.14 / 8.11.  (1024 entries a
+// row: 514 us, 1719 us, 8.30 ms.)
+constexpr int MS_WARP_ENTRIES = 24576;
 constexpr int MS_LONG_ITEMS = 1;  // entries a thread tests per long-row chunk (RMAT-24: 10.08 ms, four 10.14)
 
 #ifndef BFS_MS_PULL_R
@@ -190,6 +198,7 @@ constexpr int MS_LONG_ITEMS = 1;  // entries a thread tests per long-row chunk (
 #endif
 constexpr int MS_PULL_R = BFS_MS_PULL_R;  // in-neighbours loaded per serial pull step
 constexpr int MS_COOP_U = 4;  // 32-entry groups a warp loads per step when it finishes a long row
+
 // Words a warp takes at a time in a pull level: one while many vertices
 // still miss live lanes (costly words: finest balance).  Once few do, up to
 // 32, so that the takes don't queue on the cursor's atomics and most words are
@@ -483,6 +492,22 @@ __device__ __forceinline__ uint64_t warp_or64(uint64_t x) {
 // lane-major in a warp-uniform loop over the union of the new lanes, so the
 // 32 vertices' entries of one lane's depth row go out together.
 
+// Leaves the rows of the lanes in `rows`, from entry `from` on, to ms_long_rows.
+// Warp-uniform.
+__device__ __forceinline__ void ms_defer(const ParamsMS& p, const MsLevel& L, unsigned rows, int v,
+                                         int from) {
+    const unsigned lane = lane_id();
+    const int leader = __ffs(rows) - 1;
+    unsigned long long base = 0;
+    if ((int)lane == leader) base = atomicAdd(L.c.long_len, (unsigned long long)__popc(rows));
+    base = __shfl_sync(0xffffffffu, base, leader);
+    if ((rows >> lane) & 1u) {
+        const unsigned long long r = base + __popc(rows & lanemask_lt());
+        p.longv[r] = v;
+        p.acc_long[r] = (unsigned long long)from;  // until the CTA stores what it found
+    }
+}
+
 template <bool PAR>
 __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, MsSmem& sm, const uint64_t* f_cur) {
     const unsigned lane = lane_id();
@@ -525,14 +550,8 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
         const bool longrow = miss != 0 && end - beg > L.c.long_row;
         const unsigned lm = __ballot_sync(0xffffffffu, longrow);
         if (lm) {
-            unsigned long long base = 0;
-            const int leader = __ffs(lm) - 1;
-            if ((int)lane == leader) base = atomicAdd(L.c.long_len, (unsigned long long)__popc(lm));
-            base = __shfl_sync(0xffffffffu, base, leader);
+            ms_defer(p, L, lm, v, beg);
             if (longrow) {
-                const unsigned long long r = base + __popc(lm & lanemask_lt());
-                p.longv[r] = v;
-                p.acc_long[r] = 0;
                 miss = 0;
                 end = beg;
             }
@@ -567,6 +586,8 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
             j = min(j + MS_PULL_R, lim);  // the warp goes on from here
         }
         unsigned rm = __ballot_sync(0xffffffffu, miss != 0 && acc != miss && j < end);
+        unsigned rest = 0;           // rows the warp gives up
+        int left = MS_WARP_ENTRIES;  // entries it scans in the word's rows
         while (rm) {
             const int l = __ffs(rm) - 1;
             const int jl = __shfl_sync(0xffffffffu, j, l);
@@ -575,7 +596,8 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
             const uint64_t ml = __shfl_sync(0xffffffffu, (unsigned long long)miss, l);
             uint64_t al = __shfl_sync(0xffffffffu, (unsigned long long)acc, l);
             // MS_COOP_U * 32 entries a step: all column loads, then all mask loads
-            for (int b2 = jl; b2 < el && al != ml; b2 += 32 * MS_COOP_U) {
+            int b2 = jl;
+            for (; b2 < el && left > 0 && al != ml; b2 += 32 * MS_COOP_U, left -= 32 * MS_COOP_U) {
                 int uu[MS_COOP_U];
                 uint64_t fu[MS_COOP_U];
 #pragma unroll
@@ -613,9 +635,14 @@ __device__ void ms_pull_level(const ParamsMS& p, const UnitView& g, MsLevel& L, 
                 }
                 al |= got;
             }
-            if ((int)lane == l) acc = al;
+            if ((int)lane == l) {
+                acc = al;
+                j = b2;
+            }
+            if (al != ml && b2 < el) rest |= 1u << l;
             rm &= rm - 1;
         }
+        if (rest) ms_defer(p, L, rest, v, j);
         // depths and parents of the word, lane-major: for each lane found
         // anywhere in the word, its row entries of the 32 vertices go out
         // together.  Four lanes at a time: their parent gathers are in flight
@@ -682,7 +709,7 @@ __device__ void ms_long_rows(const ParamsMS& p, const UnitView& g, MsSmem& sm, c
     const int per = MS_LONG_ITEMS * T;
     for (long long r = blockIdx.x; r < nl; r += gridDim.x) {
         const int v = p.longv[r];
-        const int beg = __ldg(g.csc_ptr + v), end = __ldg(g.csc_ptr + v + 1);
+        const int beg = (int)p.acc_long[r], end = __ldg(g.csc_ptr + v + 1);
         const uint64_t miss = live & ~((const unsigned long long*)p.seen)[v];
         if (threadIdx.x == 0) s_or = 0;
         __syncthreads();
@@ -732,7 +759,8 @@ __device__ void ms_long_finalize(const ParamsMS& p, const UnitView& g, MsSmem& s
         const uint64_t acc = __ldcg(p.acc_long + r);
         if (!acc) continue;
         const int v = p.longv[r];
-        ((unsigned long long*)f_next)[v] = acc;
+        const uint64_t had = ((const unsigned long long*)f_next)[v];  // what the warp found, and counted
+        ((unsigned long long*)f_next)[v] = had | acc;
         const uint64_t old = ((const unsigned long long*)p.seen)[v];
         ((unsigned long long*)p.seen)[v] = old | acc;
         uint64_t b = write_depth ? acc : 0ull;
@@ -741,9 +769,11 @@ __device__ void ms_long_finalize(const ParamsMS& p, const UnitView& g, MsSmem& s
             sm.depth[j][v] = dnext;
             b &= b - 1;
         }
-        cnt += 1;
         const unsigned long long dv = (unsigned long long)(__ldg(g.row_ptr + v + 1) - __ldg(g.row_ptr + v));
-        ef += dv;
+        if (!had) {
+            cnt += 1;
+            ef += dv;
+        }
         if (((old | acc) & live) == live) done += dv;
         if ((old | acc) == g.lanes) atomicOr(p.full + (v >> 5), 1u << (v & 31));
         ln |= acc;

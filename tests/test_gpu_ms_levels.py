@@ -104,3 +104,35 @@ def test_long_rows(width, k):
                 if par and j % 9 == 0:
                     assert oracle.validate(adj, v, ref[v], parent[j].cpu().numpy()) == 0
     g.free()
+
+
+# Rows a warp gives up once it has scanned MS_WARP_ENTRIES in a word, on graphs of
+# more than two words a warp: what the warp found and what the CTA finds in the rest of the row
+# must add up (depths, parents, levels past the history, the frontier's counts).
+@pytest.mark.parametrize("width", [1024 + 32, 1024 + 33, 1700, 8192])
+@pytest.mark.parametrize("k", [3, 64])
+def test_rows_given_up(width, k):
+    from paper_2607_17106_gb300 import build
+    build.build()
+    hubs, tail, n = 200, 40, 500_000
+    rng = np.random.default_rng(width + k)
+    s = np.repeat(np.arange(hubs, dtype=np.int32), width)
+    d = (hubs + np.tile(np.arange(width), hubs)).astype(np.int32)
+    path = np.arange(hubs + width, hubs + width + tail, dtype=np.int32)  # into the last entry of every hub's row
+    s, d = np.concatenate([s, path]), np.concatenate([d, path[1:], np.int32([hubs + width - 1])])
+    adj = oracle.build_adjacency(n, s, d)
+    g = bg.Graph.build(n, s, d)
+    srcs = np.concatenate([path[[0, 20, 39]], rng.integers(0, hubs + width + tail, k - 3)]).astype(np.int32)
+    ref = {v: oracle.bfs(adj, v, with_parent=False)[0] for v in set(srcs.tolist())}
+    for o in (dict(policy=bg.BFS_POLICY_PULL), dict(policy=bg.BFS_POLICY_PULL, pull_serial=1), dict()):
+        for par in (True, False):
+            depth = torch.full((k, n), -9, dtype=torch.int32, device="cuda")
+            parent = torch.full((k, n), -9, dtype=torch.int32, device="cuda") if par else None
+            g.run(srcs, depth, parent, bg.options(batch=1, **o))
+            g.sync()
+            got = depth.cpu().numpy()
+            for j, v in enumerate(srcs.tolist()):
+                assert np.array_equal(got[j], ref[v]), (o, j)
+                if par and (j < 3 or j % 9 == 0):
+                    assert oracle.validate(adj, v, ref[v], parent[j].cpu().numpy()) == 0
+    g.free()
