@@ -41,7 +41,15 @@ namespace bfsgb {
 namespace {
 
 constexpr int ELL_T = 1024;
-constexpr long long ELL_WAIT_NS = 1000000000ll;  // a level's wait is never given up earlier
+// A level's wait is never given up earlier, whatever the caller's limit.  No
+// input makes these waits run out; a build with 0 leaves them to the caller's
+// limit alone and polls, where a try_wait sleeps in the hardware for longer than
+// a level takes.
+#ifndef BFS_SMALL_WAIT_NS
+#define BFS_SMALL_WAIT_NS 1000000000ll
+#endif
+constexpr long long ELL_WAIT_NS = BFS_SMALL_WAIT_NS;
+constexpr long long ELL_DRAIN_NS = 1000000000ll;  // limit of a failed launch's waits for the stores under way
 
 template <int W>
 struct EllCfg {
@@ -82,6 +90,9 @@ __device__ __forceinline__ void st_async(unsigned a, unsigned x, unsigned bar) {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];" ::"r"(a), "r"(x), "r"(bar)
                  : "memory");
 }
+__device__ __forceinline__ void st_cluster(unsigned a, unsigned x) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(x) : "memory");
+}
 __device__ __forceinline__ void mbar_init(unsigned long long* b, int arrivals) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"((unsigned)__cvta_generic_to_shared(b)), "r"(arrivals)
                  : "memory");
@@ -99,21 +110,30 @@ __device__ __forceinline__ bool mbar_try(unsigned bar, unsigned parity) {
     unsigned ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"
+#if BFS_SMALL_WAIT_NS > 0
         "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+#else
+        "mbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+#endif
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
         : "r"(bar), "r"(parity)
         : "memory");
     return ok != 0;
 }
-// false: the limit has passed
+// false: the limit has passed, and still nothing (this CTA may have been off
+// the GPU since its last try)
 __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity, int64_t limit_ns) {
     if (mbar_try(bar, parity)) return true;
     const uint64_t t0 = globaltimer_ns();
     while (!mbar_try(bar, parity))
-        if ((int64_t)(globaltimer_ns() - t0) > limit_ns) return false;
+        if ((int64_t)(globaltimer_ns() - t0) > limit_ns) return mbar_try(bar, parity);
     return true;
 }
+// The barrier that counts the stores of level l into the next one's queues,
+// and the parity of its phase (the two take turns).
+__device__ __forceinline__ int level_bar(int l) { return (l & 1) ^ 1; }
+__device__ __forceinline__ unsigned level_parity(int l) { return (unsigned)(l >> 1) & 1u; }
 __device__ __forceinline__ void cluster_sync() {
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -146,6 +166,7 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
     __shared__ unsigned s_cnt[2][16];                 // packed claims of each CTA, by level parity
     __shared__ unsigned s_mine[2];                    // this CTA's, being counted
     __shared__ unsigned long long s_bar[2];           // a level's arrivals and bytes, by level parity
+    __shared__ unsigned s_left[16];                   // each CTA's levels sent as it left them, bit 0: it gave up a wait
     const int cl = (int)gridDim.x, lg = __ffs(cl) - 1, rank = (int)cluster_rank();
     const int lane = (int)lane_id();
     const int grp = (int)threadIdx.x / W, j = (int)threadIdx.x % W;
@@ -187,7 +208,7 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
 
     // the counters fit in 32 bits: a CSR has less than 2^31 entries
     int level = 0, m_u = (int)p.m, f_prev = 0, f = 0, e_f = 0;
-    bool done = false;
+    bool done = false, gave_up = false;
     for (;; ++level) {
         const int par = level & 1;
         const unsigned mine = lane < cl ? s_cnt[par][lane] : 0u;
@@ -231,7 +252,7 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
                                  (rank - from) & (cl - 1), lg);
         const int32_t* q = ell_q + ((size_t)par * cl + from) * C::PART * C::PITCH;
         int32_t* qn = ell_q + ((size_t)(par ^ 1) * cl + rank) * C::PART * C::PITCH;  // this CTA's part, at any receiver
-        unsigned long long* const bar = &s_bar[par ^ 1];
+        unsigned long long* const bar = &s_bar[level_bar(level)];
         for (int i0 = 0; i0 < len; i0 += per) {  // warp-uniform
             int u = -1, w = -1;
             if (i0 + r < len) {
@@ -284,18 +305,39 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
         f_prev = f;
         bool ok = true;
         if (threadIdx.x < 32) {
-            ok = mbar_wait((unsigned)__cvta_generic_to_shared(bar), (level >> 1) & 1, limit_ns);
+            ok = mbar_wait((unsigned)__cvta_generic_to_shared(bar), level_parity(level), limit_ns);
             __syncwarp();
         }
-        if (!__syncthreads_and(ok)) {  // CTA-uniform; the other CTAs' waits end the same way
+        if (!__syncthreads_and(ok)) {  // CTA-uniform, but each CTA finds out for itself
             if (threadIdx.x == 0) atomicCAS(&ctl->bar.err, 0, (int)DEV_TIMEOUT);
-            f = 0;
-            done = true;
+            gave_up = true;
             break;
         }
     }
-    // No CTA leaves before all have stopped sending.
+    // No CTA leaves before all have stopped sending, and every CTA learns how
+    // the others left.
+    const int sent = level + (gave_up ? 1 : 0);  // levels whose stores this CTA has sent; it has waited for `level` of them
+    if (threadIdx.x < (unsigned)cl) st_cluster(map_shared(&s_left[rank], threadIdx.x), (unsigned)sent << 1 | (gave_up ? 1u : 0u));
     cluster_sync();
+    const unsigned left = lane < cl ? s_left[lane] : 0u;
+    if (__any_sync(0xffffffffu, left & 1u)) {  // cluster-uniform: the search has failed for all
+        // The cluster barrier does not order counted stores: some may still be on
+        // their way to a CTA that did not wait for them.  A CTA sends a level only
+        // when every CTA has sent the one before, so `sent` differs by one at most:
+        // who is behind arrives for that level too, without stores, and everyone
+        // waits for its own barrier up to it.
+        const int last = (int)__reduce_max_sync(0xffffffffu, left >> 1);
+        if (sent < last && threadIdx.x < (unsigned)cl) mbar_arrive_tx(map_shared(&s_bar[level_bar(last - 1)], threadIdx.x), 0u);
+        if (threadIdx.x < 32) {
+            for (int l = level; l < last; ++l)
+                mbar_wait((unsigned)__cvta_generic_to_shared(&s_bar[level_bar(l)]), level_parity(l), ELL_DRAIN_NS);
+        }
+        cluster_sync();
+        // nothing of the frontier is handed over: the CTAs have left at different levels
+        f = 0;
+        e_f = 0;
+        done = true;
+    }
     // The frontier F_level that was not expanded: depths and parents, and the
     // queue entries of the grid-wide kernel.  Nothing is left of a finished one.
     if (f > 0) {

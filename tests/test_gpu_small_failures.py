@@ -1,0 +1,88 @@
+"""What the small-level kernel does when something goes wrong.
+
+No input makes its waits run out, so the library is linked here with a copy of
+that one file that gives a wait up at the caller's limit, instead of a second
+at least.
+"""
+import contextlib
+import gc
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import graphgen
+import oracle
+import paper_2607_17106_gb300 as bg
+from paper_2607_17106_gb300 import build
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+def _link(tmp, *flags):
+    """The library with bfs_small.cu compiled with `flags`."""
+    build.build()
+    src = os.path.join(build.CSRC, "bfs_small.cu")
+    obj, lib = os.path.join(tmp, "bfs_small.o"), os.path.join(tmp, "libbfsgb_variant.so")
+    objs = [os.path.join(build.OUT_DIR, os.path.basename(s)[:-3] + ".o") for s in build.sources() if s != src]
+    nvcc = build._nvcc()
+    subprocess.run([nvcc, *build.ARCH, *build.NVCC_FLAGS, *flags, "-c", src, "-o", obj], check=True)
+    subprocess.run([nvcc, *build.ARCH, "-shared", "-o", lib, obj, *objs], check=True)
+    return lib
+
+
+@contextlib.contextmanager
+def _loaded(path):
+    kept, bg._lib = bg._lib, None
+    try:
+        yield bg.load(path)
+    finally:
+        gc.collect()  # graphs are freed by the library that made them
+        bg._lib = kept
+
+
+def _search(g, n, src, **opt):
+    depth = torch.full((n,), -9, dtype=torch.int32, device="cuda")
+    parent = torch.full((n,), -9, dtype=torch.int32, device="cuda")
+    g.run(np.array([src], np.int32), depth, parent, bg.options(batch=0, **opt))
+    g.sync()
+    return depth.cpu().numpy(), parent.cpu().numpy()
+
+
+def _graph(kind):
+    if kind == "grid":  # rows of 4
+        return graphgen.grid(161, 127, 0.1, seed=4)
+    n = 4000            # rows of 8: a ring with chords
+    v = np.arange(n, dtype=np.int32)
+    return n, np.concatenate([v, v, v]), np.concatenate([(v + 1) % n, (v + 17) % n, (v + 63) % n]).astype(np.int32)
+
+
+def test_given_up_waits(tmp_path):
+    # CTAs give up at their own times: some while others finish the level, hand
+    # the search over or find it done.  The call reports it, or succeeds with the
+    # right depths, and the next search on the same graph is right.
+    lib = _link(str(tmp_path), "-DBFS_SMALL_WAIT_NS=0")
+    with _loaded(lib):
+        for kind in ("grid", "ring"):
+            n, s, d = _graph(kind)
+            adj = oracle.build_adjacency(n, s, d)
+            g = bg.Graph.build(n, s, d)
+            rng = np.random.default_rng(7)
+            timeouts = {}
+            for limit in (1, 200, 400, 600, 800, 1000, 1500, 2000, 4000, 1000000):
+                timeouts[limit] = 0
+                for src in rng.integers(0, n, 12):
+                    ref, _ = oracle.bfs(adj, int(src), with_parent=False)
+                    # gamma: with 1e-6 only the frontier's size ends the cluster's part
+                    for gamma in (16.0, 1e-6):
+                        try:
+                            assert np.array_equal(_search(g, n, int(src), barrier_timeout_ns=limit, gamma=gamma)[0], ref)
+                        except bg.BfsError as e:
+                            assert e.status == bg.BFS_ETIMEOUT
+                            timeouts[limit] += 1
+                depth, parent = _search(g, n, int(src))
+                assert np.array_equal(depth, ref) and oracle.validate(adj, int(src), depth, parent) == 0
+            g.free()
+            assert timeouts[1] > 0
