@@ -436,8 +436,8 @@ int ell_cluster() {
 int ell_width(int32_t deg_max) { return deg_max <= 4 ? 4 : deg_max <= 8 ? 8 : 0; }
 
 // Rows of ell_width entries in w->ell, made once per workspace.  False: no
-// memory for them, or the stream is being captured (no allocation there); the
-// search then takes the general kernel.
+// memory for them, they could not be launched, or the stream is being captured
+// (no allocation there); the search then takes the general kernel.
 bool ell_prepare(const bfs_graph* g, Workspace1* w, cudaStream_t st) {
     if (w->ell) return true;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
@@ -451,9 +451,17 @@ bool ell_prepare(const bfs_graph* g, Workspace1* w, cudaStream_t st) {
         w->ell = nullptr;
         return false;
     }
-    const int64_t blocks = std::min<int64_t>(div_up((int64_t)g->n * width, 256), (int64_t)num_sms() * 32);
-    ell_build_kernel<<<(unsigned)blocks, 256, 0, st>>>(g->row_ptr, g->col, g->n, width, w->ell);
-    return true;  // a failed launch shows at the search's own
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)std::min<int64_t>(div_up((int64_t)g->n * width, 256), (int64_t)num_sms() * 32));
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    if (cudaLaunchKernelEx(&cfg, ell_build_kernel, (const int32_t*)g->row_ptr, (const int32_t*)g->col, g->n, width,
+                           w->ell) == cudaSuccess)
+        return true;
+    cudaGetLastError();
+    cudaFree(w->ell);
+    w->ell = nullptr;  // never rows that were not written: their entries are used as vertices
+    return false;
 }
 
 // Rows are loaded with the candidates while they fit in L2 (126 MB): on a

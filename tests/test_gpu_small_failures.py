@@ -1,10 +1,12 @@
 """What the small-level kernel does when something goes wrong.
 
-No input makes its waits run out, so the library is linked here with a copy of
-that one file that gives a wait up at the caller's limit, instead of a second
-at least.
+No input makes its waits run out or its launches fail, so the library is linked
+here with a copy of that one file that gives a wait up at the caller's limit
+(instead of a second at least), or whose first launch is refused by a fake of
+the runtime's call.
 """
 import contextlib
+import ctypes
 import gc
 import os
 import subprocess
@@ -20,6 +22,17 @@ from paper_2607_17106_gb300 import build
 torch = pytest.importorskip("torch")
 
 pytestmark = pytest.mark.gpu
+
+FAKE = """
+#include <cuda_runtime.h>
+extern "C" { int fake_launches = 0; }
+template <typename K, typename... A>
+static cudaError_t fake_launch(const cudaLaunchConfig_t* c, K k, A... a) {
+    return fake_launches++ == 0 ? cudaErrorLaunchOutOfResources : cudaLaunchKernelEx(c, k, a...);
+}
+#define cudaLaunchKernelEx fake_launch
+"""
+
 
 def _link(tmp, *flags):
     """The library with bfs_small.cu compiled with `flags`."""
@@ -86,3 +99,23 @@ def test_given_up_waits(tmp_path):
                 assert np.array_equal(depth, ref) and oracle.validate(adj, int(src), depth, parent) == 0
             g.free()
             assert timeouts[1] > 0
+
+
+def test_rows_that_could_not_be_launched(tmp_path):
+    fake = tmp_path / "fake.h"
+    fake.write_text(FAKE)
+    lib = _link(str(tmp_path), "-include", str(fake))
+    with _loaded(lib) as handle:
+        launches = ctypes.c_int.in_dll(handle, "fake_launches")
+        n, s, d = _graph("grid")
+        adj = oracle.build_adjacency(n, s, d)
+        g = bg.Graph.build(n, s, d)
+        seen = []
+        for src in (5, 700, 9000):
+            ref, _ = oracle.bfs(adj, src, with_parent=False)
+            depth, parent = _search(g, n, src)
+            assert np.array_equal(depth, ref) and oracle.validate(adj, src, depth, parent) == 0
+            seen.append(launches.value)
+        g.free()
+        # refused: the general kernel; then the rows and the search; then the search
+        assert seen == [1, 3, 4]
