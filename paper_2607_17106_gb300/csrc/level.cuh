@@ -1054,20 +1054,42 @@ constexpr int PULL_LPI = 2;
 // 14.83 ms, two 14.38, three 14.3, four 14.6; RMAT-22 8.67, 8.51, 8.53, 8.67).
 constexpr int PULL_R2 = 2;
 
-// Next-queue entries of the vertices a pull level found (symmetric graphs: the
-// in-row bounds are the row's).  Warp-uniform.
-__device__ __forceinline__ void append_found(const Params1& p, LevelCtx& L, bool found, int v, int beg, int end) {
-    const unsigned m = __ballot_sync(0xffffffffu, found);
-    if (!m) return;
-    unsigned long long base = 0;
-    if (lane_id() == 0) base = atomicAdd(&L.next->q_len, (unsigned long long)__popc(m));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (base + (unsigned long long)__popc(m) > (unsigned long long)L.qcap) {
-        if (lane_id() == 0) atomicCAS(L.err, 0, (int)DEV_OVERFLOW);
-    } else if (found) {
-        L.q_next[base + __popc(m & lanemask_lt())] = make_int4(v, beg, end, 0);
+// Next-queue entries of the vertices a pull level found in word wl of each
+// lane.  Their row bounds are read again (from L2, a round of the level's end):
+// appending inside the scan, where they are in registers, made its long-row loop
+// slower in every pull level (BFS_POLICY_PULL, 4 sources, ms, there / here: RMAT-18
+// 3.71 / 2.88, RMAT-22 135 / 130; by the direction test RMAT-22 is 16 sources 2.04
+// either way, 2.07 without appending).  Warp-uniform.
+__device__ __forceinline__ void append_words(const Params1& p, LevelCtx& L, unsigned found, long long wl) {
+    const int c = __popc(found);
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, o);
+        if ((int)lane_id() >= o) incl += y;
     }
-    emit_units_warp(p, L.u_next, L.next, found && end - beg >= p.chunk, v, end - beg);
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    if (total == 0) return;
+    unsigned long long base = 0;
+    if (lane_id() == 0) base = atomicAdd(&L.next->q_len, (unsigned long long)total);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (base + (unsigned long long)total > (unsigned long long)L.qcap) {
+        if (lane_id() == 0) atomicCAS(L.err, 0, (int)DEV_OVERFLOW);
+        return;
+    }
+    unsigned long long at = base + (unsigned long long)(incl - c);
+    while (__any_sync(0xffffffffu, found != 0)) {
+        const bool has = found != 0;
+        int v = 0, rb = 0, re = 0;
+        if (has) {
+            v = (int)(wl * 32 + __ffs(found) - 1);
+            rb = __ldg(p.row_ptr + v);
+            re = __ldg(p.row_ptr + v + 1);
+            L.q_next[at++] = make_int4(v, rb, re, 0);
+            found &= found - 1;
+        }
+        emit_units_warp(p, L.u_next, L.next, has && re - rb >= p.chunk, v, re - rb);
+    }
 }
 
 // Scans of up to PULL_LPI listed vertices per lane (v < 0: none), as in
@@ -1183,7 +1205,6 @@ __device__ __forceinline__ void pull_list_scan(const Params1& p, LevelCtx& L, un
             }
             rm &= rm - 1;
         }
-        if (L.append) append_found(p, L, found[q], v[q], beg[q], end[q]);
         if (found[q]) {
             atomicOr(nb + sl[q], 1u << (v[q] & 31));
             L.depth[v[q]] = L.level + 1;
@@ -1277,11 +1298,12 @@ __device__ void pull_level_list(const Params1& p, LevelCtx& L, const uint32_t* f
             pull_list_scan<NC, T == 1024>(p, L, ls.nb, f_cur, v, sl, serial);
         }
         __syncthreads();
+        const unsigned nb = own ? ls.nb[slot] : 0u;
         if (own) {
-            const unsigned nb = ls.nb[slot];
             f_next[wl] = nb;
             if (nb) p.P[wl] = pwl | nb;
         }
+        if (L.append) append_words(p, L, nb, wl);
     }
 }
 
