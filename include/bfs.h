@@ -169,9 +169,11 @@ enum {
  * after it, runs in the full persistent kernel (a second launch on the same
  * stream, no host round trip).  Sources run one launch pair each.
  * BFS_SMALL_AUTO also runs whole searches of small graphs of higher degree (up
- * to about 49,000 vertices with an edge and 2 million entries) in the cluster,
- * in one launch, unless the launch shape is set or barrier_timeout_ns is below
- * a millisecond (the hardware barrier takes no limit). */
+ * to about 49,000 vertices with an edge and 2 million entries, 786,000 without a
+ * hub) in the cluster, in one launch, where the direction test pulls the dense
+ * levels (BFS_POLICY_HEURISTIC or _MLP near the default thresholds; any policy up
+ * to 131,000 entries).  Not if the launch shape is set or barrier_timeout_ns is
+ * below its default: the hardware barrier takes no limit. */
 enum {
     BFS_SMALL_AUTO = -1, /* on for graphs whose maximum degree is at most 16 (grids, road-like graphs) */
     BFS_SMALL_OFF = 0,
@@ -214,7 +216,8 @@ typedef struct {
     int32_t block_threads;   /* threads per CTA of the persistent single-source kernel: 256, 512 or 1024 (1024) */
     int32_t blocks_per_sm;   /* CTAs per SM, 0 = as many as fit (persistent/cooperative launch) */
     int32_t claim_aggregate; /* push: warp-aggregate the visited-bitmap OR by word (0) */
-    int64_t barrier_timeout_ns; /* limit of one device-side wait before BFS_ETIMEOUT (2e9) */
+    int64_t barrier_timeout_ns; /* limit of one device-side wait before BFS_ETIMEOUT (2e9).  The hardware barrier of a
+                                thread-block cluster takes none, see small_levels */
     const int8_t* schedule;  /* host array for BFS_POLICY_SCHEDULE */
     int32_t schedule_len;
     int32_t max_levels;      /* stop with BFS_ERANGE after this many levels, 0 = n + 1 */

@@ -36,6 +36,7 @@
 // graphs a launch of one thread-block cluster runs the small levels first
 // and the grid-wide launch continues from its saved state.
 #include "level.cuh"
+#include "small_rule.h"
 
 #include <algorithm>
 #include <cmath>
@@ -512,6 +513,7 @@ int max_coop_blocks(int blocks_per_sm) {
 // Small levels (bfs_options.small_levels): one cluster of 1024-thread CTAs,
 // 16 where the GPU can co-schedule such a cluster, else 8 (0: none).
 constexpr int SMALL_T = 1024;
+static_assert(SMALL_THREADS == 16 * SMALL_T, "the threads that the rule counts with");
 static int small_cluster_size() {
     static int cached[64] = {};
     const int d = device_id();
@@ -574,24 +576,12 @@ static int small_levels_for(const bfs_graph* g, const bfs_options& o) {
     return small_cluster_size();
 }
 
-// Whole searches in the cluster: up to three vertices with an edge for each
-// of its threads.  A level's barrier and counter read take 0.7 us there, 2.0
-// grid-wide, and the launch is cheaper; above, 16 SMs fall behind.  One search,
-// us, grid-wide / cluster: RMAT-10 34.6 / 29.0, RMAT-14 45.4 / 41.4, RMAT-16 (46,000
-// vertices with an edge) 51.1 / 46.8, RMAT-17 57.0 / 60.8; ER of degree 16: 16,384
-// vertices 45.4 / 41.4, 32,768 50.2 / 47.9, 65,536 53.5 / 57.7.
-// The hardware barrier takes no limit: a call that limits its waits to less
-// than such a search may take gets the grid-wide kernel, as does one that asks
-// for a launch shape or no cluster.
-constexpr int64_t SMALL_GRAPH_N = 3 * 16 * SMALL_T, SMALL_GRAPH_M = 1 << 21, SMALL_GRAPH_WAIT_NS = 1000000;
+// Whole searches in the cluster (small_rule.h).  The cluster size, 0 for no.
 static int small_graph_for(const bfs_graph* g, const bfs_options& o) {
     bfs_options d;
     bfs_options_init(&d);
-    if (o.mode != BFS_MODE_PERSISTENT || o.frontier_sort != BFS_SORT_NONE || o.push_filter != BFS_PUSH_FUSED) return 0;
-    if (o.small_levels != BFS_SMALL_AUTO || o.block_threads != d.block_threads || o.blocks_per_sm != 0) return 0;
-    if (g->n - g->n_isolated > SMALL_GRAPH_N || g->m > SMALL_GRAPH_M || g->n > 4 * SMALL_GRAPH_N) return 0;
-    if (o.barrier_timeout_ns < SMALL_GRAPH_WAIT_NS || g->deg_max <= 16) return 0;
-    return small_cluster_size();
+    const SmallGraph sg{g->n, (int64_t)g->n - g->n_isolated, g->m, g->deg_max};
+    return small_graph_pays(sg, o, d) ? small_cluster_size() : 0;
 }
 
 static cudaError_t run_small_graph(Params1 q, int cl, cudaStream_t st) {
