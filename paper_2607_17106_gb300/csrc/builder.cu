@@ -557,11 +557,14 @@ __global__ void __launch_bounds__(256)
 }
 
 // One allocation for everything a build needs while it runs.  Large ones by
-// cudaMalloc: 2 GB from the stream-ordered pool cost 1.7 ms to map and 3 ms to
-// trim at the next synchronisation, cudaMalloc and cudaFree 0.9 ms.  Up to
-// 32 MB, the least the pool maps, from the pool: builds that follow one
-// another find it still mapped (117 us by cudaMalloc), if it is given back
-// after the last wait of a build (a wait trims the pool: 45 us).
+// cudaMalloc: 1.1 GB from the stream-ordered pool costs 0.9 to 1.1 ms to map and
+// 1.5 ms to trim at the next synchronisation.  They go back by cudaFreeAsync,
+// in the stream's order (0.6 ms, paid in the stream's next wait): cudaFree, 0.45
+// ms, waits for the work of every stream, and a build beside a search on another
+// stream waited for that too.  Up to 32 MB, the least the pool maps, from the
+// pool: builds that follow one another find it still mapped (117 us by
+// cudaMalloc), if it is given back after the last wait of a build (a wait trims
+// the pool: 45 us).
 struct Arena {
     cudaStream_t st;
     unsigned char* base = nullptr;
@@ -586,8 +589,7 @@ struct Arena {
         return p;
     }
     void drop() {
-        if (base && pooled()) cudaFreeAsync(base, st);
-        else cudaFree(base);
+        if (base) cudaFreeAsync(base, st);
         base = nullptr;
         need = used = 0;
     }
@@ -1099,7 +1101,18 @@ extern "C" bfs_status bfs_build_graph(int32_t n, int64_t m, const int32_t* src, 
     }
     take_rows(g, r, sym);
     g->symmetric = sym;
-    if (!ar.pooled() || (flags & (BFS_REORDER_RCM | BFS_PULL_HUBS_FIRST))) ar.drop();
+    const bool more = (flags & (BFS_REORDER_RCM | BFS_PULL_HUBS_FIRST)) != 0;
+    if (!ar.pooled()) {
+        ar.drop();
+        // back before the steps below take theirs (they wait too)
+        const cudaError_t e = more ? cudaStreamSynchronize(st) : cudaSuccess;
+        if (e != cudaSuccess) {
+            bfs_free_graph(g);
+            return cuda_fail(e, "build scratch");
+        }
+    } else if (more) {
+        ar.drop();
+    }
     if (sym && (flags & BFS_REORDER_RCM)) {
         bfs_status sr = rcm_reorder(g, bits, st);
         if (sr != BFS_OK) {
