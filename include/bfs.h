@@ -216,8 +216,9 @@ typedef struct {
     int32_t block_threads;   /* threads per CTA of the persistent single-source kernel: 256, 512 or 1024 (1024) */
     int32_t blocks_per_sm;   /* CTAs per SM, 0 = as many as fit (persistent/cooperative launch) */
     int32_t claim_aggregate; /* push: warp-aggregate the visited-bitmap OR by word (0) */
-    int64_t barrier_timeout_ns; /* limit of one device-side wait before BFS_ETIMEOUT (2e9).  The hardware barrier of a
-                                thread-block cluster takes none, see small_levels */
+    int64_t barrier_timeout_ns; /* limit of one device-side wait before BFS_ETIMEOUT (2e9).  Where small levels run in a
+                                thread-block cluster: one second at least on graphs of maximum degree <= 8; the
+                                hardware barrier of the other cluster launches takes no limit (see BFS_SMALL_*) */
     const int8_t* schedule;  /* host array for BFS_POLICY_SCHEDULE */
     int32_t schedule_len;
     int32_t max_levels;      /* stop with BFS_ERANGE after this many levels, 0 = n + 1 */

@@ -48,7 +48,8 @@ int msbfs_sticky_error(bfs_graph* g);  // msbfs.cu
 bfs_status run_graph_mode(bfs_graph* g, Workspace1* w, Params1& p, int32_t src, int32_t* depth, int32_t* parent,
                           const bfs_options& o, cudaStream_t st);  // bfs_graph.cu
 
-int ell_width(int32_t deg_max);  // bfs_small.cu
+int64_t small_wait_ns(int64_t timeout_ns);  // bfs_small.cu
+int ell_width(int32_t deg_max);
 int ell_cluster_size(const bfs_graph* g, int width);
 bool ell_prepare(const bfs_graph* g, Workspace1* w, cudaStream_t st);
 cudaError_t ell_launch(const bfs_graph* g, Params1 p, int width, int cl, cudaStream_t st);
@@ -683,6 +684,8 @@ static bfs_status ensure_ws1(bfs_graph* g, int32_t chunk, cudaStream_t st, Works
 
 bfs_status device_error(int err, int64_t timeout_ns) {
     if (err == DEV_TIMEOUT) return fail(BFS_ETIMEOUT, "grid barrier wait exceeded %lld ns", (long long)timeout_ns);
+    if (err == DEV_TIMEOUT_SMALL)
+        return fail(BFS_ETIMEOUT, "small level's wait exceeded %lld ns", (long long)small_wait_ns(timeout_ns));
     if (err == DEV_OVERFLOW) return fail(BFS_EVALIDATE, "device work list overflow");
     if (err == DEV_LEVELS) return fail(BFS_ERANGE, "level limit exceeded");
     return fail(BFS_EVALIDATE, "device error %d", err);
@@ -698,7 +701,7 @@ bfs_status sync_graph(bfs_graph* g, cudaStream_t st) {
         if (err) BFS_CUDA(cudaMemset(g->ws1->d_sticky, 0, 4));
     }
     if (!err) err = msbfs_sticky_error(g);
-    if (err) return device_error(err, 0);
+    if (err) return device_error(err, g->wait_ns);
     return BFS_OK;
 }
 

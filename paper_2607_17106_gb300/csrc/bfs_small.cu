@@ -173,7 +173,6 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
     const int per = C::GROUPS / cl;            // groups that expand the entries of one sender
     const int from = grp / per, r = grp % per; // warp-uniform sender: per * W >= 32
     Ctl1* ctl = p.ctl;
-    const int64_t limit_ns = max((long long)p.timeout_ns, ELL_WAIT_NS);
 
     if (threadIdx.x < 32) {
         const int s = p.src_value;
@@ -305,11 +304,11 @@ __global__ void __launch_bounds__(ELL_T, 1) bfs_small_kernel(Params1 p) {
         f_prev = f;
         bool ok = true;
         if (threadIdx.x < 32) {
-            ok = mbar_wait((unsigned)__cvta_generic_to_shared(bar), level_parity(level), limit_ns);
+            ok = mbar_wait((unsigned)__cvta_generic_to_shared(bar), level_parity(level), p.timeout_ns);
             __syncwarp();
         }
         if (!__syncthreads_and(ok)) {  // CTA-uniform, but each CTA finds out for itself
-            if (threadIdx.x == 0) atomicCAS(&ctl->bar.err, 0, (int)DEV_TIMEOUT);
+            if (threadIdx.x == 0) atomicCAS(&ctl->bar.err, 0, (int)DEV_TIMEOUT_SMALL);
             gave_up = true;
             break;
         }
@@ -433,6 +432,9 @@ int ell_cluster() {
 
 }  // namespace
 
+// Limit of a level's waits for a caller's limit
+int64_t small_wait_ns(int64_t timeout_ns) { return std::max<int64_t>(timeout_ns, ELL_WAIT_NS); }
+
 int ell_width(int32_t deg_max) { return deg_max <= 4 ? 4 : deg_max <= 8 ? 8 : 0; }
 
 // Rows of ell_width entries in w->ell, made once per workspace.  False: no
@@ -483,6 +485,7 @@ int ell_cluster_size(const bfs_graph* g, int width) {
 // vertices, the outputs -1 and the control block zeros.
 cudaError_t ell_launch(const bfs_graph* g, Params1 p, int width, int cl, cudaStream_t st) {
     const bool spec = ell_speculate(g, width);
+    p.timeout_ns = small_wait_ns(p.timeout_ns);
     cudaLaunchAttribute attr[1];
     if (width == 4) {
         p.small_ef_max = ell_max_frontier<4>(cl);

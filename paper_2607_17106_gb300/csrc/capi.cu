@@ -152,6 +152,7 @@ extern "C" bfs_status bfs_run(const bfs_graph* gc, const int32_t* sources, int32
         if (src[j] < 0 || src[j] >= g->n) return fail(BFS_EINVAL, "source %d = %d outside [0, %d)", j, src[j], g->n);
     const float* mlp = (o.policy == BFS_POLICY_MLP) ? policy_device_weights(o.mlp) : nullptr;
     std::lock_guard<std::mutex> lk(g->lock);
+    g->wait_ns = o.barrier_timeout_ns;
     bool dev_out = is_device_ptr(depth) && (!parent || is_device_ptr(parent));
     if (k > 1 && o.batch) {
         return run_msbfs(g, src.data(), k, depth, parent, o, mlp, st);

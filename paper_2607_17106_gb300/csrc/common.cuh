@@ -31,7 +31,8 @@ enum : int32_t {
     DEV_OK = 0,
     DEV_TIMEOUT = 1,     // a grid/team barrier wait exceeded its limit
     DEV_OVERFLOW = 2,    // a work list exceeded its capacity
-    DEV_LEVELS = 3       // max_levels exceeded
+    DEV_LEVELS = 3,      // max_levels exceeded
+    DEV_TIMEOUT_SMALL = 4  // a small level's wait for its stores exceeded its limit (bfs_small.cu)
 };
 
 // ------------------------------------------------------------------ graph
@@ -58,6 +59,7 @@ struct bfs_graph {
     double deg_mean = 0, deg_var = 0;
     void* cc_scratch = nullptr;   // bfs_components: control block and row list (cc.cu), made on first use
     std::mutex lock;
+    int64_t wait_ns = 0;  // limit of the last run's device-side waits, for the message of an asynchronous failure
     bfsgb::Workspace1* ws1 = nullptr;
     bfsgb::WorkspaceMS* wsms = nullptr;
     // bfs_run_mixed: the workspace of the calls whose largest graph this is, and

@@ -93,7 +93,7 @@ def test_given_up_waits(tmp_path):
                         try:
                             assert np.array_equal(_search(g, n, int(src), barrier_timeout_ns=limit, gamma=gamma)[0], ref)
                         except bg.BfsError as e:
-                            assert e.status == bg.BFS_ETIMEOUT
+                            assert e.status == bg.BFS_ETIMEOUT and f"exceeded {limit} ns" in str(e)
                             timeouts[limit] += 1
                 depth, parent = _search(g, n, int(src))
                 assert np.array_equal(depth, ref) and oracle.validate(adj, int(src), depth, parent) == 0
@@ -119,3 +119,16 @@ def test_rows_that_could_not_be_launched(tmp_path):
         g.free()
         # refused: the general kernel; then the rows and the search; then the search
         assert seen == [1, 3, 4]
+
+
+def test_message_names_the_limit():
+    # of the run that failed, also where bfs_sync reports it
+    build.build()
+    n, s, d = graphgen.rmat(14, 16, seed=1)
+    g = bg.Graph.build(n, s, d)
+    for k, opt in ((1, dict(batch=0)), (3, dict(batch=0)), (3, dict(batch=1))):
+        depth = torch.empty((k, n), dtype=torch.int32, device="cuda")
+        with pytest.raises(bg.BfsError) as e:
+            g.run(s[:k], depth, None, bg.options(barrier_timeout_ns=7, **opt))
+            g.sync()
+        assert e.value.status == bg.BFS_ETIMEOUT and "exceeded 7 ns" in str(e.value)
