@@ -1215,11 +1215,18 @@ static int64_t count_units(bfs_graph* g, int32_t chunk, cudaStream_t st) {
     unsigned long long* d = nullptr;
     unsigned long long h = 0;
     if (cudaMallocAsync(&d, 8, st) != cudaSuccess) return -1;
-    cudaMemsetAsync(d, 0, 8, st);
-    ms_count_units_kernel<<<num_sms() * 8, 256, 0, st>>>(g->row_ptr, g->n, chunk, d);
-    cudaMemcpyAsync(&h, d, 8, cudaMemcpyDeviceToHost, st);
+    cudaError_t e = cudaMemsetAsync(d, 0, 8, st);
+    if (e == cudaSuccess) {
+        ms_count_units_kernel<<<num_sms() * 8, 256, 0, st>>>(g->row_ptr, g->n, chunk, d);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d, 8, cudaMemcpyDeviceToHost, st);
     cudaFreeAsync(d, st);
-    if (cudaStreamSynchronize(st) != cudaSuccess) return -1;
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        return -1;  // and nothing is kept: a count of 0 would refuse every later batch
+    }
     g->units_chunk = chunk;
     g->units_count = (int64_t)h;
     return (int64_t)h;

@@ -1,9 +1,9 @@
-"""What the small-level kernel does when something goes wrong.
+"""What the library does when a wait runs out or a runtime call fails.
 
-No input makes its waits run out or its launches fail, so the library is linked
-here with a copy of that one file that gives a wait up at the caller's limit
-(instead of a second at least), or whose first launch is refused by a fake of
-the runtime's call.
+No input makes the small levels' waits run out, the launch of their rows fail or
+a copy fail, so the library is linked here with a copy of one file that gives a
+wait up at the caller's limit (instead of a second at least), or whose first
+launch or copy is refused by a fake of the runtime's call.
 """
 import contextlib
 import ctypes
@@ -23,22 +23,30 @@ torch = pytest.importorskip("torch")
 
 pytestmark = pytest.mark.gpu
 
-FAKE = """
+FAKE_LAUNCH = """
 #include <cuda_runtime.h>
-extern "C" { int fake_launches = 0; }
+extern "C" { int fake_calls = 0; }
 template <typename K, typename... A>
 static cudaError_t fake_launch(const cudaLaunchConfig_t* c, K k, A... a) {
-    return fake_launches++ == 0 ? cudaErrorLaunchOutOfResources : cudaLaunchKernelEx(c, k, a...);
+    return fake_calls++ == 0 ? cudaErrorLaunchOutOfResources : cudaLaunchKernelEx(c, k, a...);
 }
 #define cudaLaunchKernelEx fake_launch
 """
+FAKE_COPY = """
+#include <cuda_runtime.h>
+extern "C" { int fake_calls = 0; }
+static cudaError_t fake_copy(void* d, const void* s, size_t n, cudaMemcpyKind k, cudaStream_t st) {
+    return fake_calls++ == 0 ? cudaErrorInvalidValue : cudaMemcpyAsync(d, s, n, k, st);
+}
+#define cudaMemcpyAsync fake_copy
+"""
 
 
-def _link(tmp, *flags):
-    """The library with bfs_small.cu compiled with `flags`."""
+def _link(tmp, name, *flags):
+    """The library with csrc/`name` compiled with `flags`."""
     build.build()
-    src = os.path.join(build.CSRC, "bfs_small.cu")
-    obj, lib = os.path.join(tmp, "bfs_small.o"), os.path.join(tmp, "libbfsgb_variant.so")
+    src = os.path.join(build.CSRC, name)
+    obj, lib = os.path.join(tmp, "variant.o"), os.path.join(tmp, "libbfsgb_variant.so")
     objs = [os.path.join(build.OUT_DIR, os.path.basename(s)[:-3] + ".o") for s in build.sources() if s != src]
     nvcc = build._nvcc()
     subprocess.run([nvcc, *build.ARCH, *build.NVCC_FLAGS, *flags, "-c", src, "-o", obj], check=True)
@@ -76,7 +84,7 @@ def test_given_up_waits(tmp_path):
     # CTAs give up at their own times: some while others finish the level, hand
     # the search over or find it done.  The call reports it, or succeeds with the
     # right depths, and the next search on the same graph is right.
-    lib = _link(str(tmp_path), "-DBFS_SMALL_WAIT_NS=0")
+    lib = _link(str(tmp_path), "bfs_small.cu", "-DBFS_SMALL_WAIT_NS=0")
     with _loaded(lib):
         for kind in ("grid", "ring"):
             n, s, d = _graph(kind)
@@ -103,10 +111,10 @@ def test_given_up_waits(tmp_path):
 
 def test_rows_that_could_not_be_launched(tmp_path):
     fake = tmp_path / "fake.h"
-    fake.write_text(FAKE)
-    lib = _link(str(tmp_path), "-include", str(fake))
+    fake.write_text(FAKE_LAUNCH)
+    lib = _link(str(tmp_path), "bfs_small.cu", "-include", str(fake))
     with _loaded(lib) as handle:
-        launches = ctypes.c_int.in_dll(handle, "fake_launches")
+        launches = ctypes.c_int.in_dll(handle, "fake_calls")
         n, s, d = _graph("grid")
         adj = oracle.build_adjacency(n, s, d)
         g = bg.Graph.build(n, s, d)
@@ -132,3 +140,24 @@ def test_message_names_the_limit():
             g.run(s[:k], depth, None, bg.options(barrier_timeout_ns=7, **opt))
             g.sync()
         assert e.value.status == bg.BFS_ETIMEOUT and "exceeded 7 ns" in str(e.value)
+
+
+def test_unit_count_that_failed(tmp_path):
+    # a batch's chunk units are counted once per graph; a count that failed is
+    # reported and not kept
+    fake = tmp_path / "fake.h"
+    fake.write_text(FAKE_COPY)
+    lib = _link(str(tmp_path), "msbfs.cu", "-include", str(fake))
+    with _loaded(lib):
+        n, s, d = graphgen.rmat(13, 16, seed=1)
+        adj = oracle.build_adjacency(n, s, d)
+        g = bg.Graph.build(n, s, d)
+        depth = torch.full((5, n), -9, dtype=torch.int32, device="cuda")
+        run = lambda: bg.run_mixed([g], [0] * 5, s[:5], list(depth), opt=bg.options(chunk=64))  # noqa: E731
+        with pytest.raises(bg.BfsError) as e:
+            run()
+        assert e.value.status == bg.BFS_ECUDA
+        run()
+        for j in range(5):
+            assert np.array_equal(depth[j].cpu().numpy(), oracle.bfs(adj, int(s[j]), with_parent=False)[0])
+        g.free()
