@@ -70,7 +70,8 @@ enum {
  * src/dst: host or device, not modified.  *out receives a new graph, freed
  * with bfs_free_graph.  Errors: EINVAL (null pointer, n <= 0, m < 0, id
  * outside [0, n)), ERANGE (more than 2^31-1 directed entries before or after
- * deduplication), ENOMEM, ECUDA.  Synchronises `cuda_stream`.
+ * deduplication), ENOMEM, ECUDA.  Synchronises `cuda_stream` (BFS_REORDER_RCM
+ * the device).
  *
  * BFS_REORDER_RCM: the paper reorders every input with Reverse Cuthill-McKee
  * (Section 7.1).  Vertices are ranked by (degree, id) in the symmetric, built
@@ -163,11 +164,18 @@ enum {
 
 /* Small levels of a single-source search (persistent drive).  While a push
  * level's frontier is small, one thread-block cluster (16 CTAs where the GPU
- * can co-schedule them, else 8) runs the levels with the cluster's hardware
- * barrier instead of the grid-wide barrier; the first level that would pull
- * or that has more frontier edges than the cluster's threads, and every level
- * after it, runs in the full persistent kernel (a second launch on the same
- * stream, no host round trip).  Sources run one launch pair each.
+ * can co-schedule them, else 8) runs the levels without grid-wide barriers; the
+ * first level that would pull, read the bitmap or is too large for the cluster,
+ * and every level after it, runs in the full persistent kernel (a second launch
+ * on the same stream, no host round trip).  Sources run one launch pair each.
+ * Graphs of maximum degree <= 8 (BFS_POLICY_HEURISTIC and _PUSH): a level's CTAs
+ * wait for its messages on a barrier in shared memory, whose limit is
+ * barrier_timeout_ns but one second at least; too large is a frontier of more than
+ * about 16,000 vertices (degree <= 4) or 4,900 (degree <= 8).  The first such search
+ * makes rows of 4 or 8 neighbours that stay with the graph (16 or 32 bytes a
+ * vertex, freed with it; without memory for them the search runs without).
+ * Other graphs: the cluster's hardware barrier, without a limit; too large is more
+ * frontier edges than the cluster has threads.
  * BFS_SMALL_AUTO also runs whole searches of small graphs of higher degree (up
  * to about 49,000 vertices with an edge and 2 million entries, 786,000 without a
  * hub) in the cluster, in one launch, where the direction test pulls the dense
@@ -272,8 +280,8 @@ bfs_status bfs_sync(const bfs_graph* g, void* cuda_stream);
  * parent[q] (each an int32 array of that graph's n; device memory).
  * graph_of_query/sources are host arrays of length nq; graphs has n_graphs
  * entries; depth/parent are host arrays of nq device pointers (parent or its
- * entries may be NULL).  Queries are grouped per graph into 64-lane units and
- * the units are handed out to CTA teams by a device work counter.
+ * entries may be NULL).  Queries are grouped per graph into 64-lane units, and
+ * the launch runs one unit after another on the whole GPU.
  * The workspace (about 200 bytes a vertex of the largest graph in the batch)
  * stays with that graph and is freed with it; a call that finds it in use by
  * another thread's call makes its own.

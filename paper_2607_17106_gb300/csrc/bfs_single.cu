@@ -884,7 +884,8 @@ bfs_status run_single(bfs_graph* g, int32_t src_value, int32_t* depth, int32_t* 
 
 // k sources, one search after another, all in ONE persistent launch (device
 // outputs [k][n], persistent drive, no level log): the per-search launch and
-// control-block reset are paid once.  A barrier separates the searches.
+// control-block reset are paid once.  No barrier separates two searches (see the
+// end of bfs1_body's loop over them).
 bfs_status run_single_many(bfs_graph* g, const int32_t* src_host, int32_t k, int32_t* depth, int32_t* parent,
                            const bfs_options& o, const float* mlp_dev, cudaStream_t st) {
     Workspace1* w;

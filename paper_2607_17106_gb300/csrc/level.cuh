@@ -123,7 +123,7 @@ struct Params1 {
     int32_t level_count;  // levels to run in this launch (host loop: 1)
     int64_t small_ef_max; // cluster launch: leave before a level with more frontier edges (bfs_small.cu: vertices) or a pull
     int32_t small_whole;  // cluster launch: every level, whatever its form and size
-    int32_t rows_filled;  // the -1 of the depth and parent rows was stored before the launch (else when the search ends)
+    int32_t rows_filled;  // the -1 of the depth and parent rows was stored before the launch (else as the search starts)
 };
 
 // ------------------------------------------------------------- direction

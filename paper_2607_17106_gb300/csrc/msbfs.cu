@@ -208,8 +208,9 @@ constexpr int MS_COOP_U = 4;  // 32-entry groups a warp loads per step when it f
 constexpr int MS_PULL_CHUNK = 32, MS_PULL_TAKES = 4;
 
 // A level's constants.  These and the unit's live in shared memory: at 64
-// registers a thread (two CTAs an SM) they were spilled, and the spills were
-// 170 million memory requests of an RMAT-22 batch.
+// registers a thread (two CTAs an SM) they were spilled, and those spills were 170
+// million memory requests of an RMAT-22 batch.  (140 bytes of other state are
+// still spilled, 148 without parents.)
 struct MsLevelConst {
     int32_t level;
     int pull_chunk;              // pull: words a warp takes at a time

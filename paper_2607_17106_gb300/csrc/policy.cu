@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(128) mlp_forward_kernel(const float* __restric
 // ------------------------------------------------------------ training
 constexpr int TR_T = 128;         // threads of a training CTA
 constexpr int TR_W = TR_T / 32;
-constexpr int TR_PER_SM = 2;      // resident CTAs (about 200 registers a thread)
+constexpr int TR_PER_SM = 2;      // resident CTAs (244 registers a thread, 255 with the softmax)
 constexpr int TR_LD = 36;         // row pitch of the staged activations: 16-byte stores of 8 lanes then hit 8 bank groups
 constexpr int NPART = NPARAM + 1; // a CTA's partial gradient, then its share of the loss
 
