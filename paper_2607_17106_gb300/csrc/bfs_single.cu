@@ -255,7 +255,12 @@ __device__ __forceinline__ void bfs1_body(const Params1& p) {
         q_valid = __ldcg(&ctl->q_valid);
         m_u = (int)__ldcg(&ctl->m_u);
         f_prev = (int)__ldcg(&ctl->f_prev);
-        done = __ldcg(&ctl->done) != 0;
+        // A launch that finds the search finished sets `done` with no barrier behind
+        // the other CTAs' reads (the rest of the state stays as it was).  A CTA that
+        // sees it early leaves, as it would have anyway, but all its threads alike:
+        // when each went by its own read, thread 0 could leave before others went
+        // into a level whose counters it had not loaded for them.
+        done = __syncthreads_or(__ldcg(&ctl->done) != 0) != 0;
     }
     const int level_end = level + p.level_count;
 
